@@ -229,8 +229,9 @@ tnmc_status tnmc_env_status(const tnmc_env* env, int32_t* status);
  * energy      device double [B] (output)
  * flags       device int32 [B] or NULL (output; TNMC_FLAG_NUMERIC)
  * The first call on an env may allocate device scratch for the per-sample
- * right-vector stacks (grown, never shrunk, freed with the env).  FP64/FP32:
- * (Lx+1) * P * 64 * 8 or (Lx+1) * P * 128 * 4 bytes per resident CTA.  BF16
+ * right-vector stacks (grown, never shrunk, freed with the env).  FP64:
+ * (Lx+1) * P * 8 bytes, FP32: (Lx+1) * Q * 4 bytes per resident sample (Q: P rounded up
+ * to the output blocks, at most 4/3 P).  BF16
  * (tensor cores, chi <= 64): Lx * 32 KiB per resident CTA, e.g. 2.5 GB for
  * Lx = 256 on a 152-SM GPU; the BF16 path also reads the pre-swizzled operand
  * tiles derived at build time (64 KiB per site).

@@ -81,6 +81,18 @@ bool is_integer_array(const double* p, size_t n) {
   return true;
 }
 
+// Exponent of the fixed-point couplings: the largest magnitude times the number of terms of
+// H stays below 2^61 units.
+int fixed_point_exponent(const tnmc_lattice& lat, size_t nJh, size_t nJv, size_t nh) {
+  double mx = 0.0;
+  for (size_t i = 0; i < nJh; ++i) mx = fmax(mx, fabs(lat.Jh[i]));
+  for (size_t i = 0; i < nJv; ++i) mx = fmax(mx, fabs(lat.Jv[i]));
+  for (size_t i = 0; i < nh; ++i) mx = fmax(mx, fabs(lat.h[i]));
+  if (mx == 0.0) return 0;
+  const int terms = ilogb((double)(nJh + nJv + nh)) + 1;
+  return ilogb(mx) + 1 + terms - 61;
+}
+
 }  // namespace
 
 namespace {
@@ -128,11 +140,14 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
     return o;
   };
   const size_t oJh = take((nJh ? nJh : 1) * 8), oJv = take((nJv ? nJv : 1) * 8), oh = take(nh * 8);
+  const size_t oqJh = take((nJh ? nJh : 1) * 8), oqJv = take((nJv ? nJv : 1) * 8), oqh = take(nh * 8);
+  const size_t ocoup = off;   // the coupling arrays above are uploaded as one image
   const size_t ofe = take(nh * 2 * 8), ofe32 = take(nh * 2 * 4);
   const size_t obond = take((size_t)Ly * (Lx + 1) * 4), oesz = take((size_t)Ly * (Lx + 1) * 4);
   const size_t oM64 = take(tens * 8), oR64 = take(tens * 8);
   const size_t oL32 = (mask & (1 << TNMC_F32)) ? take(tens * 4) : 0;
   const size_t oR32 = (mask & (1 << TNMC_F32)) ? take(tens * 4) : 0;
+  const size_t oK32 = (mask & (1 << TNMC_F32)) ? take(tens * 4) : 0;
   const size_t oL16 = (mask & (1 << TNMC_BF16)) ? take(ntens * tnmc_tc_tile_bytes()) : 0;
   const size_t oR16 = (mask & (1 << TNMC_BF16)) ? take(ntens * tnmc_tc_tile_bytes()) : 0;
   const size_t oh32 = take(nh * 4), oJh32 = take((nJh ? nJh : 1) * 4), oJv32 = take((nJv ? nJv : 1) * 4);
@@ -182,6 +197,7 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
   d.R64 = reinterpret_cast<const double*>(base + oR64);
   d.L32 = oL32 ? reinterpret_cast<const float*>(base + oL32) : nullptr;
   d.R32 = oR32 ? reinterpret_cast<const float*>(base + oR32) : nullptr;
+  d.K32 = oK32 ? reinterpret_cast<const float*>(base + oK32) : nullptr;
   d.L16 = oL16 ? reinterpret_cast<const __nv_bfloat16*>(base + oL16) : nullptr;
   d.R16 = oR16 ? reinterpret_cast<const __nv_bfloat16*>(base + oR16) : nullptr;
   d.status = reinterpret_cast<int32_t*>(base + ostat);
@@ -194,12 +210,32 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
   env->Jh32 = reinterpret_cast<float*>(base + oJh32);
   env->Jv32 = reinterpret_cast<float*>(base + oJv32);
 
+  d.qJh = reinterpret_cast<const int64_t*>(base + oqJh);
+  d.qJv = reinterpret_cast<const int64_t*>(base + oqJv);
+  d.qh = reinterpret_cast<const int64_t*>(base + oqh);
+  std::vector<char> image;
   tnmc_status st = TNMC_OK;
+  try {
+    image.resize(ocoup);
+  } catch (const std::bad_alloc&) {
+    dev_free(env->alloc, base, total, s);
+    delete env;
+    tnmc_set_error("host allocation failed");
+    return TNMC_E_NOMEM;
+  }
+  d.qexp = fixed_point_exponent(*lat, nJh, nJv, nh);
+  auto put = [&](const double* src, size_t cnt, size_t o, size_t oq) {
+    if (cnt == 0) return;
+    memcpy(image.data() + o, src, cnt * 8);
+    int64_t* q = reinterpret_cast<int64_t*>(image.data() + oq);
+    for (size_t i = 0; i < cnt; ++i) q[i] = llrint(ldexp(src[i], -d.qexp));
+  };
+  put(lat->Jh, nJh, oJh, oqJh);
+  put(lat->Jv, nJv, oJv, oqJv);
+  put(lat->h, nh, oh, oqh);
   do {
     if (cudaMemsetAsync(base, 0, total, s) != cudaSuccess) { st = TNMC_E_CUDA; break; }
-    if (nJh && cudaMemcpyAsync(const_cast<double*>(d.Jh), lat->Jh, nJh * 8, cudaMemcpyHostToDevice, s) != cudaSuccess) { st = TNMC_E_CUDA; break; }
-    if (nJv && cudaMemcpyAsync(const_cast<double*>(d.Jv), lat->Jv, nJv * 8, cudaMemcpyHostToDevice, s) != cudaSuccess) { st = TNMC_E_CUDA; break; }
-    if (cudaMemcpyAsync(const_cast<double*>(d.h), lat->h, nh * 8, cudaMemcpyHostToDevice, s) != cudaSuccess) { st = TNMC_E_CUDA; break; }
+    if (cudaMemcpyAsync(base, image.data(), ocoup, cudaMemcpyHostToDevice, s) != cudaSuccess) { st = TNMC_E_CUDA; break; }
     // the host arrays may be released as soon as this call returns
     if (cudaStreamSynchronize(s) != cudaSuccess) { st = TNMC_E_CUDA; break; }
   } while (0);

@@ -26,7 +26,8 @@
 
 #include "common.cuh"
 #include "metropolis_kernel.cuh"
-#include "sample_simt_kernel.cuh"
+#include "sample_f32_kernel.cuh"
+#include "sample_f64_kernel.cuh"
 
 namespace tnmc {
 namespace {
@@ -67,26 +68,60 @@ __device__ __forceinline__ uint64_t global_ns() {
 
 // cta_ns[2 i], cta_ns[2 i + 1]: when CTA i started and when it found no item left (global
 // timer, ns): the load balance of the launch is sum(busy) / (grid x makespan).
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) sample_batched_kernel(const SampleArgs<T>* __restrict__ tab,
-                                                            const int2* __restrict__ items, int64_t nitems,
-                                                            unsigned int* counter, T* scratch, size_t stack_elems,
-                                                            uint64_t* cta_ns) {
-  extern __shared__ unsigned char smem_raw[];
+// FP32: a CTA of NW warps takes an item at a time, NW 8 SB samples at once.
+template <int SB, int XBM>
+__global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM))
+    sample_batched_f32_kernel(const SampleArgs<float>* __restrict__ tab, const int2* __restrict__ items, int64_t nitems,
+                              int tile, unsigned long long* counter, float* scratch, size_t stack_elems,
+                              uint64_t* cta_ns) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int2 item;
-  T* stack = scratch + (size_t)blockIdx.x * stack_elems;
+  __shared__ SampleArgs<float> a;
+  const int step = (blockDim.x >> 5) * (8 * SB);
+  float* stack = scratch + (size_t)blockIdx.x * stack_elems * step;
   if (threadIdx.x == 0) cta_ns[2 * blockIdx.x] = global_ns();
   for (;;) {
     if (threadIdx.x == 0) {
-      const unsigned int k = atomicAdd(counter, 1u);
-      item = (k < (uint64_t)nitems) ? items[k] : make_int2(-1, -1);
+      const unsigned long long k = atomicAdd(counter, 1ull);
+      item = (k < (unsigned long long)nitems) ? items[k] : make_int2(-1, -1);
     }
     __syncthreads();
     const int2 it = item;
     __syncthreads();
     if (it.x < 0) break;
-    const SampleArgs<T> a = tab[it.x];
-    sample_simt_tile<T, NT>(a, it.y, smem_raw, stack);
+    {
+      const int* src = reinterpret_cast<const int*>(tab + it.x);
+      for (int q = threadIdx.x; q < (int)(sizeof(a) / sizeof(int)); q += blockDim.x) reinterpret_cast<int*>(&a)[q] = src[q];
+    }
+    __syncthreads();
+    for (int64_t base = (int64_t)it.y * tile; base < (int64_t)(it.y + 1) * tile && base < a.B; base += step)
+      sample_f32_tile<SB, XBM>(a, base, smem_raw, stack);
+  }
+  if (threadIdx.x == 0) cta_ns[2 * blockIdx.x + 1] = global_ns();
+}
+
+// FP64: one warp per CTA.  A work item of `tile` samples is handed out in tile / S warp tiles
+// (consecutive counter values), so that a batch of few samples still spreads over every SM.
+template <int LS, int SB>
+__global__ void __launch_bounds__(32, kF64MinWarps) sample_batched_f64_kernel(const SampleArgs<double>* __restrict__ tab,
+                                                                const int2* __restrict__ items, int64_t nitems,
+                                                                int tile, unsigned long long* counter,
+                                                                double* scratch, size_t stack_elems,
+                                                                uint64_t* cta_ns) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int S = LS * SB;
+  const int per = tile / S;
+  double* stack = scratch + (size_t)blockIdx.x * stack_elems * S;
+  if (threadIdx.x == 0) cta_ns[2 * blockIdx.x] = global_ns();
+  for (;;) {
+    unsigned long long k = 0;
+    if (threadIdx.x == 0) k = atomicAdd(counter, 1ull);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    if (k >= (unsigned long long)nitems * per) break;
+    const int2 it = items[k / per];
+    const SampleArgs<double> a = tab[it.x];
+    const int64_t base = (int64_t)it.y * tile + (int64_t)(k % per) * S;
+    if (base < a.B) sample_f64_tile<LS, SB>(a, base, smem_raw, stack);
   }
   if (threadIdx.x == 0) cta_ns[2 * blockIdx.x + 1] = global_ns();
 }
@@ -229,7 +264,11 @@ struct tnmc_batch {
   int64_t prop_rows = 0, prop_bytes = 0, chain_rows = 0, chain_bytes = 0;
   int64_t items_prop = 0, items_chain = 0;
   int grid = 0;
-  size_t smem = 0, stack_elems = 0, scratch_bytes = 0, arena_bytes = 0;
+  size_t smem = 0, stack_elems = 0, scratch_bytes = 0, arena_bytes = 0;   // stack_elems: per sample
+  int max_P = 1;
+  // samples per warp, warps per CTA and shared memory of the proposal [0] and chain [1] launches
+  int s_warp[2] = {0, 0}, warps[2] = {1, 1};
+  size_t smem_of[2] = {0, 0};
   tnmc::Allocator alloc;   // the hook current when the plan was created
   // device memory: one arena for the tables, one for the per-CTA stacks
   void* arena = nullptr;
@@ -245,7 +284,7 @@ struct tnmc_batch {
   tnmc::MhInst* d_mh = nullptr;
   tnmc::MetroInst* d_metro = nullptr;
   int max_sites = 0;
-  unsigned int* d_counter = nullptr;
+  unsigned long long* d_counter = nullptr;
   uint64_t* d_params = nullptr;
   int64_t* d_last = nullptr;
   uint64_t* d_cta_ns = nullptr;   // [grid][2] timers of the last sampling launch
@@ -260,7 +299,7 @@ const T* env_L(const tnmc_env* e);
 template <>
 const double* env_L<double>(const tnmc_env* e) { return e->d.M64; }
 template <>
-const float* env_L<float>(const tnmc_env* e) { return e->d.L32; }
+const float* env_L<float>(const tnmc_env* e) { return e->d.K32; }
 template <typename T>
 const T* env_R(const tnmc_env* e);
 template <>
@@ -274,29 +313,72 @@ const double* env_fe<double>(const tnmc_env* e) { return e->d.fe; }
 template <>
 const float* env_fe<float>(const tnmc_env* e) { return e->d.fe32; }
 
-template <typename T, int NT>
-tnmc_status plan_kernel_setup(tnmc_batch* p, int max_P, int max_W) {
+template <class F>
+tnmc_status by_f64_tile(int S, F&& f) {
+  using tnmc::IntC;
+  switch (S) {
+    case 32: return f(IntC<8>{}, IntC<4>{});
+    case 16: return f(IntC<8>{}, IntC<2>{});
+    case 8: return f(IntC<8>{}, IntC<1>{});
+    case 4: return f(IntC<4>{}, IntC<1>{});
+    default: return f(IntC<2>{}, IntC<1>{});
+  }
+}
+
+// The tile shapes of the proposal and the chain launches, and a grid for both.
+tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
   using namespace tnmc;
-  auto kern = sample_batched_kernel<T, NT>;
-  p->smem = (size_t)3 * max_P * NT * sizeof(T) + (size_t)2 * max_W * NT * sizeof(uint32_t);
   int dev = 0, nsm = 0, max_optin = 0;
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (p->smem + sizeof(int2) > (size_t)max_optin) {
-    tnmc_set_error("batched sampler needs %zu bytes of shared memory per CTA (device allows %d)", p->smem, max_optin);
-    return TNMC_E_UNSUPPORTED;
+  const bool f64 = p->precision == TNMC_F64;
+  int64_t grid = 1;
+  size_t samples = 0;      // largest CTA tile
+  for (int q = 0; q < 2; ++q) {
+    const int64_t rows = q ? p->chain_rows : p->prop_rows;
+    int64_t tiles = 0;       // CTA tiles that hold samples: more CTAs than that would leave SMs uneven
+    int S, NW = 1, per_sm = 0;
+    tnmc_status st;
+    if (f64) {
+      S = f64_tile_samples(rows, p->max_P, nsm);
+      const size_t smem = f64_tile_smem(p->max_P, max_Lx, S);
+      p->smem_of[q] = smem;
+      st = by_f64_tile(S, [&](auto ls, auto sb) -> tnmc_status {
+        auto kern = sample_batched_f64_kernel<decltype(ls)::value, decltype(sb)::value>;
+        if (smem > 48 * 1024) TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem));
+        return TNMC_OK;
+      });
+    } else {
+      const int SB = f32_block(rows, p->max_P, nsm);
+      S = 8 * SB;
+      NW = f32_warps(p->max_P, max_Lx, SB, std::max(1, std::min(4, p->tile / S)), (size_t)max_optin - 1024);
+      if (NW == 0) {
+        tnmc_set_error("batched sampler needs %zu bytes of shared memory per CTA (device allows %d)",
+                       f32_smem(p->max_P, max_Lx, SB, 1).total, max_optin);
+        return TNMC_E_UNSUPPORTED;
+      }
+      const size_t smem = f32_smem(p->max_P, max_Lx, SB, NW).total;
+      p->smem_of[q] = smem;
+      st = by_f32_block(SB, p->max_P, [&](auto sb, auto xbm) -> tnmc_status {
+        auto kern = sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value>;
+        TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, smem));
+        return TNMC_OK;
+      });
+    }
+    if (st != TNMC_OK) return st;
+    p->s_warp[q] = S;
+    p->warps[q] = NW;
+    const int64_t unit = f64 ? S : p->tile;
+    for (int i = 0; i < p->n; ++i) tiles += ((q ? p->chains : p->B[i]) + unit - 1) / unit;
+    grid = std::max(grid, std::min<int64_t>(tiles, (int64_t)nsm * std::max(per_sm, 1)));
+    samples = std::max(samples, (size_t)S * NW);
   }
-  TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
-  int per_sm = 0;
-  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, p->smem));
-  if (per_sm < 1) per_sm = 1;
-  int64_t grid = (int64_t)nsm * per_sm;
-  const int64_t most = std::max(p->items_prop, p->items_chain);
-  if (grid > most) grid = most;
-  if (grid < 1) grid = 1;
+  p->smem = std::max(p->smem_of[0], p->smem_of[1]);
   p->grid = (int)grid;
-  p->scratch_bytes = (size_t)grid * p->stack_elems * sizeof(T);
+  p->scratch_bytes = (size_t)grid * p->stack_elems * samples * (f64 ? sizeof(double) : sizeof(float));
   return TNMC_OK;
 }
 
@@ -315,34 +397,51 @@ void fill_table(const tnmc_batch* p, std::vector<SampleArgs<T>>& tab, bool chain
   }
 }
 
-template <typename T, int NT>
-tnmc_status launch_batched(tnmc_batch* p, bool chains, const int8_t* spins_in, int8_t* spins_out, double* logq,
-                           double* energy, int32_t* flags, cudaStream_t s) {
+// The per-call fields of the plan's sampler arguments, and a fresh item counter.
+template <typename T>
+tnmc_status batched_begin(tnmc_batch* p, bool chains, const int8_t* spins_in, int8_t* spins_out, double* logq,
+                          double* energy, int32_t* flags, cudaStream_t s) {
   using namespace tnmc;
-  const int64_t nitems = chains ? p->items_chain : p->items_prop;
-  if (nitems == 0) return TNMC_OK;
   auto* tab = static_cast<SampleArgs<T>*>(chains ? p->tab_chain : p->tab_prop);
   const int64_t* row = chains ? p->d_chain_row : p->d_prop_row;
   const int64_t* spin = chains ? p->d_chain_spin : p->d_prop_spin;
   batch_prepare_kernel<T><<<(p->n + 127) / 128, 128, 0, s>>>(tab, p->n, row, spin, p->d_params, spins_in,
                                                              spins_out, logq, energy, flags);
   TNMC_CUDA_TRY(cudaGetLastError());
-  unsigned int* counter = p->d_counter + (chains ? 1 : 0);
-  TNMC_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned int), s));
-  sample_batched_kernel<T, NT><<<p->grid, NT, p->smem, s>>>(tab, chains ? p->d_items_chain : p->d_items_prop, nitems,
-                                                            counter, static_cast<T*>(p->scratch), p->stack_elems,
-                                                            p->d_cta_ns);
-  TNMC_CUDA_TRY(cudaGetLastError());
+  TNMC_CUDA_TRY(cudaMemsetAsync(p->d_counter + (chains ? 1 : 0), 0, sizeof(unsigned long long), s));
   return TNMC_OK;
 }
 
 tnmc_status dispatch_batched(tnmc_batch* p, bool chains, const int8_t* spins_in, int8_t* spins_out, double* logq,
                              double* energy, int32_t* flags, cudaStream_t s) {
-  if (p->precision == TNMC_F64)
-    return p->tile == 64 ? launch_batched<double, 64>(p, chains, spins_in, spins_out, logq, energy, flags, s)
-                         : launch_batched<double, 128>(p, chains, spins_in, spins_out, logq, energy, flags, s);
-  return p->tile == 64 ? launch_batched<float, 64>(p, chains, spins_in, spins_out, logq, energy, flags, s)
-                       : launch_batched<float, 128>(p, chains, spins_in, spins_out, logq, energy, flags, s);
+  using namespace tnmc;
+  const int q = chains ? 1 : 0;
+  const int64_t nitems = chains ? p->items_chain : p->items_prop;
+  if (nitems == 0) return TNMC_OK;
+  const void* tab = chains ? p->tab_chain : p->tab_prop;
+  const int2* items = chains ? p->d_items_chain : p->d_items_prop;
+  const int S = p->s_warp[q], threads = 32 * p->warps[q];
+  const size_t smem = p->smem_of[q];
+  if (p->precision == TNMC_F64) {
+    const tnmc_status st = batched_begin<double>(p, chains, spins_in, spins_out, logq, energy, flags, s);
+    if (st != TNMC_OK) return st;
+    return by_f64_tile(S, [&](auto ls, auto sb) -> tnmc_status {
+      sample_batched_f64_kernel<decltype(ls)::value, decltype(sb)::value><<<p->grid, threads, smem, s>>>(
+          static_cast<const SampleArgs<double>*>(tab), items, nitems, p->tile, p->d_counter + q,
+          static_cast<double*>(p->scratch), p->stack_elems, p->d_cta_ns);
+      TNMC_CUDA_TRY(cudaGetLastError());
+      return TNMC_OK;
+    });
+  }
+  const tnmc_status st = batched_begin<float>(p, chains, spins_in, spins_out, logq, energy, flags, s);
+  if (st != TNMC_OK) return st;
+  return by_f32_block(S / 8, p->max_P, [&](auto sb, auto xbm) -> tnmc_status {
+    sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value><<<p->grid, threads, smem, s>>>(
+        static_cast<const SampleArgs<float>*>(tab), items, nitems, p->tile, p->d_counter + q,
+        static_cast<float*>(p->scratch), p->stack_elems, p->d_cta_ns);
+    TNMC_CUDA_TRY(cudaGetLastError());
+    return TNMC_OK;
+  });
 }
 
 #define CHECK_ARG(cond, ...)       \
@@ -401,7 +500,7 @@ tnmc_status tnmc_batch_create(int n, tnmc_env* const* envs, const int64_t* B, in
   p->prop_spin.resize(n);
   p->chain_row.resize(n);
   p->chain_spin.resize(n);
-  int max_P = 1, max_W = 1;
+  int max_Lx = 1;
   size_t max_stack = 1;
   std::vector<double> cost(n);
   std::vector<tnmc::MhInst> mh(n);
@@ -419,9 +518,9 @@ tnmc_status tnmc_batch_create(int n, tnmc_env* const* envs, const int64_t* B, in
     p->chain_bytes += chains * ns;
     p->items_prop += (B[i] + tile - 1) / tile;
     p->items_chain += (chains + tile - 1) / tile;
-    max_P = std::max(max_P, d.P);
-    max_W = std::max(max_W, (d.Lx + 31) / 32);
-    max_stack = std::max(max_stack, (size_t)(d.Lx + 1) * d.P * tile);
+    p->max_P = std::max(p->max_P, d.P);
+    max_Lx = std::max(max_Lx, d.Lx);
+    max_stack = std::max(max_stack, precision == TNMC_F64 ? (size_t)(d.Lx + 1) * d.P : tnmc::f32_stack_floats(d.P, d.Lx));
     cost[i] = instance_cost(d);
     mh[i] = tnmc::MhInst{d.beta, ns, B[i] / chains, p->prop_row[i], p->prop_spin[i], p->chain_spin[i]};
     metro[i] = tnmc::MetroInst{d.Jh, d.Jv, d.h, d.beta, d.Lx, d.Ly, p->chain_spin[i]};
@@ -447,11 +546,7 @@ tnmc_status tnmc_batch_create(int n, tnmc_env* const* envs, const int64_t* B, in
   };
   const std::vector<int2> ip = make_items(false), ic = make_items(true);
 
-  tnmc_status st = (precision == TNMC_F64)
-                       ? (tile == 64 ? plan_kernel_setup<double, 64>(p, max_P, max_W)
-                                     : plan_kernel_setup<double, 128>(p, max_P, max_W))
-                       : (tile == 64 ? plan_kernel_setup<float, 64>(p, max_P, max_W)
-                                     : plan_kernel_setup<float, 128>(p, max_P, max_W));
+  tnmc_status st = plan_setup(p, max_Lx);
   if (st != TNMC_OK) {
     delete p;
     return st;
@@ -466,7 +561,7 @@ tnmc_status tnmc_batch_create(int n, tnmc_env* const* envs, const int64_t* B, in
   const size_t o_tp = take(tab_bytes), o_tc = take(tab_bytes);
   const size_t o_pr = take(n * 8), o_ps = take(n * 8), o_cr = take(n * 8), o_cs = take(n * 8);
   const size_t o_ip = take(ip.size() * sizeof(int2)), o_ic = take(ic.size() * sizeof(int2));
-  const size_t o_mh = take(n * sizeof(tnmc::MhInst)), o_cnt = take(2 * sizeof(unsigned int));
+  const size_t o_mh = take(n * sizeof(tnmc::MhInst)), o_cnt = take(2 * sizeof(unsigned long long));
   const size_t o_metro = take(n * sizeof(tnmc::MetroInst));
   const size_t o_par = take(2 * sizeof(uint64_t)), o_last = take((size_t)p->chain_rows * 8);
   const size_t o_ns = take((size_t)p->grid * 2 * sizeof(uint64_t));
@@ -494,7 +589,7 @@ tnmc_status tnmc_batch_create(int n, tnmc_env* const* envs, const int64_t* B, in
   p->d_items_chain = reinterpret_cast<int2*>(base + o_ic);
   p->d_mh = reinterpret_cast<tnmc::MhInst*>(base + o_mh);
   p->d_metro = reinterpret_cast<tnmc::MetroInst*>(base + o_metro);
-  p->d_counter = reinterpret_cast<unsigned int*>(base + o_cnt);
+  p->d_counter = reinterpret_cast<unsigned long long*>(base + o_cnt);
   p->d_params = reinterpret_cast<uint64_t*>(base + o_par);
   p->d_last = reinterpret_cast<int64_t*>(base + o_last);
   p->d_cta_ns = reinterpret_cast<uint64_t*>(base + o_ns);

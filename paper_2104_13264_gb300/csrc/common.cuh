@@ -17,6 +17,7 @@ constexpr int kMaxPad = 64;       // padded bond stride P <= 64
 //   M64   FP64 master, [Ly][Lx][P][2][P]  M[a][s][b]      (left layout)
 //   L{T}  sampler copy in precision T, same layout as M64
 //   R{T}  sampler copy in precision T, [Ly][Lx][P][P][2]  MT[b][a][s]
+//   K32   FP32 copy of L32 with the spins innermost, [Ly][Lx][P][P][2]  M[a][b][s]
 //   L16 / R16 (BF16) instead hold the tensor-core operand tiles: per (r, c) two
 //         128 x 64 K-major 128-byte-swizzled tiles, hi = bf16(M) then
 //         lo = bf16(M - hi) (left: n = s*64 + b, k = a; right: n = s*64 + a, k = b),
@@ -42,8 +43,15 @@ struct DeviceEnv {
   const double* R64;
   const float* L32;
   const float* R32;
+  const float* K32;
   const __nv_bfloat16* L16;
   const __nv_bfloat16* R16;
+  // couplings in 64-bit fixed point, J = q 2^qexp with |H| < 2^61 2^qexp: the energy of a
+  // configuration is an exact integer sum (integer couplings stay exact)
+  const int64_t* qJh;
+  const int64_t* qJv;
+  const int64_t* qh;
+  int qexp;
   int32_t* status;       // device status word
 };
 

@@ -2,31 +2,31 @@
 // App. A) in FP64 or FP32, and the kernel that derives the sampler copies of the
 // environment.
 //
-// One thread owns one sample.  For every row r it
+// For every row r a sample
 //   (right sweep) builds R_{Lx} = 1, R_c = sum_s f_c(s) M_c[:, s, :] R_{c+1}
 //                 for c = Lx-1 .. 1, each rescaled by a power of two and pushed
-//                 to a per-thread stack in global scratch;
+//                 to a stack in global scratch;
 //   (left sweep)  walks c = 0 .. Lx-1:  U[s] = Lambda_c M_c[:, s, :],
 //                 w(s) = f_c(s) <U[s], R_{c+1}>, clamps at 0, normalises,
 //                 draws the spin from the 64-bit Philox word (or reads it in
-//                 forced mode), accumulates log q and the energy, and sets
+//                 forced mode), accumulates log q, and sets
 //                 Lambda_{c+1} = f_c(s) U[s], rescaled by a power of two.
 // f_c(s) = exp(beta Jv[r-1][c] s_{r-1,c} s) carries the (exactly contracted)
-// product state of the rows above.  Environment tensors are read through the
-// read-only cache: every thread of a CTA reads the same element at the same
-// time, so each load is a broadcast.  Per-thread vectors live in shared memory
-// laid out [k][thread] (conflict free).
+// product state of the rows above.  On the odd rows of the snake order the two sweeps
+// change roles (draws from the right).  The kernels are in sample_f64_kernel.cuh and
+// sample_f32_kernel.cuh.
 #include <math.h>
 
 #include "common.cuh"
-#include "sample_simt_kernel.cuh"
+#include "sample_f32_kernel.cuh"
+#include "sample_f64_kernel.cuh"
 
 namespace tnmc {
 namespace {
 
-// Sampler copies: L (same layout as M64), R ([b][a][s]) and the field table.
+// Sampler copies: L (same layout as M64), R ([b][a][s]), K ([a][b][s]) and the field table.
 template <typename T>
-__global__ void derive_kernel(DeviceEnv e, T* L, T* R, size_t ntens) {
+__global__ void derive_kernel(DeviceEnv e, T* L, T* R, T* K, size_t ntens) {
   const int P = e.P;
   const size_t per = (size_t)P * 2 * P;
   const size_t total = ntens * per;
@@ -37,6 +37,7 @@ __global__ void derive_kernel(DeviceEnv e, T* L, T* R, size_t ntens) {
     const T v = (T)e.M64[i];
     if (L) L[i] = v;
     R[t * per + ((size_t)b * P + aa) * 2 + s] = v;
+    if (K) K[t * per + ((size_t)aa * P + b) * 2 + s] = v;
   }
 }
 
@@ -57,51 +58,53 @@ __global__ void fields_kernel(DeviceEnv e, double* fe, float* fe32) {
   }
 }
 
-template <typename T, int NT>
-tnmc_status launch_sample_t(const tnmc_env* env, const T* L, const T* R, const T* fe, int64_t B,
-                            uint64_t seed, uint64_t offset, const int8_t* spins_in, int8_t* spins_out,
-                            double* logq, double* energy, int32_t* flags, cudaStream_t stream) {
+// FP64: one warp per CTA, S samples per warp (f64_tile_samples).
+template <int LS, int SB>
+tnmc_status launch_sample_f64(const tnmc_env* env, SampleArgs<double> a, int nsm, cudaStream_t stream) {
+  constexpr int S = LS * SB;
   const DeviceEnv& d = env->d;
-  const int W = (d.Lx + 31) / 32;
-  const size_t smem = (size_t)3 * d.P * NT * sizeof(T) + (size_t)2 * W * NT * sizeof(uint32_t);
-  auto kern = sample_simt_kernel<T, NT>;
-  int dev = 0, nsm = 0, max_optin = 0;
-  TNMC_CUDA_TRY(cudaGetDevice(&dev));
-  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (smem > (size_t)max_optin) {
-    tnmc_set_error("sampler needs %zu bytes of shared memory per CTA (device allows %d)", smem, max_optin);
+  auto kern = sample_f64_kernel<LS, SB>;
+  const size_t smem = f64_tile_smem(d.P, d.Lx, S);
+  if (smem > 48 * 1024) TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem));
+  if (per_sm < 1) per_sm = 1;
+  int64_t grid = (a.B + S - 1) / S;
+  if (grid > (int64_t)nsm * per_sm) grid = (int64_t)nsm * per_sm;
+  tnmc_env* me = const_cast<tnmc_env*>(env);
+  const tnmc_status gs = grow_scratch(me, (size_t)grid * (d.Lx + 1) * d.P * S * sizeof(double), stream, "sampler");
+  if (gs != TNMC_OK) return gs;
+  a.scratch = static_cast<double*>(me->scratch.ptr);
+  kern<<<(unsigned)grid, 32, smem, stream>>>(a);
+  TNMC_CUDA_TRY(cudaGetLastError());
+  return TNMC_OK;
+}
+
+// FP32: CTAs of up to 4 warps, 8 SB samples per warp (f32_block).
+template <int SB, int XBM>
+tnmc_status launch_sample_f32(const tnmc_env* env, SampleArgs<float> a, int nsm, int max_smem, cudaStream_t stream) {
+  const DeviceEnv& d = env->d;
+  auto kern = sample_f32_kernel<SB, XBM>;
+  const int NW = f32_warps(d.P, d.Lx, SB, 4, (size_t)max_smem);
+  if (NW == 0) {
+    tnmc_set_error("sampler needs %zu bytes of shared memory per CTA (device allows %d)",
+                   f32_smem(d.P, d.Lx, SB, 1).total, max_smem);
     return TNMC_E_UNSUPPORTED;
   }
+  const size_t smem = f32_smem(d.P, d.Lx, SB, NW).total;
   TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
+  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, smem));
   if (per_sm < 1) per_sm = 1;
-  const int64_t ntiles = (B + NT - 1) / NT;
-  int64_t grid = (int64_t)nsm * per_sm;
-  if (grid > ntiles) grid = ntiles;
-  if (grid < 1) grid = 1;
-  const size_t need = (size_t)grid * (d.Lx + 1) * d.P * NT * sizeof(T);
+  const int64_t tile = (int64_t)NW * 8 * SB;
+  int64_t grid = (a.B + tile - 1) / tile;
+  if (grid > (int64_t)nsm * per_sm) grid = (int64_t)nsm * per_sm;
   tnmc_env* me = const_cast<tnmc_env*>(env);
-  {
-    const tnmc_status gs = grow_scratch(me, need, stream, "sampler");
-    if (gs != TNMC_OK) return gs;
-  }
-  SampleArgs<T> a;
-  a.e = d;
-  a.L = L;
-  a.Rt = R;
-  a.fe = fe;
-  a.B = B;
-  a.seed = seed;
-  a.offset = offset;
-  a.spins_in = spins_in;
-  a.spins_out = spins_out;
-  a.logq = logq;
-  a.energy = energy;
-  a.flags = flags;
-  a.scratch = static_cast<T*>(me->scratch.ptr);
-  kern<<<(unsigned)grid, NT, smem, stream>>>(a);
+  const tnmc_status gs =
+      grow_scratch(me, (size_t)grid * tile * f32_stack_floats(d.P, d.Lx) * sizeof(float), stream, "sampler");
+  if (gs != TNMC_OK) return gs;
+  a.scratch = static_cast<float*>(me->scratch.ptr);
+  kern<<<(unsigned)grid, 32 * NW, smem, stream>>>(a);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }
@@ -115,10 +118,11 @@ tnmc_status tnmc_launch_derive(tnmc_env* env, int mask, cudaStream_t stream) {
   const size_t ntens = (size_t)d.Lx * d.Ly;
   fields_kernel<<<256, 256, 0, stream>>>(d, const_cast<double*>(d.fe), const_cast<float*>(d.fe32));
   TNMC_CUDA_TRY(cudaGetLastError());
-  derive_kernel<double><<<1024, 256, 0, stream>>>(d, nullptr, const_cast<double*>(d.R64), ntens);
+  derive_kernel<double><<<1024, 256, 0, stream>>>(d, nullptr, const_cast<double*>(d.R64), nullptr, ntens);
   TNMC_CUDA_TRY(cudaGetLastError());
   if (mask & (1 << TNMC_F32)) {
-    derive_kernel<float><<<1024, 256, 0, stream>>>(d, const_cast<float*>(d.L32), const_cast<float*>(d.R32), ntens);
+    derive_kernel<float><<<1024, 256, 0, stream>>>(d, const_cast<float*>(d.L32), const_cast<float*>(d.R32),
+                                                   const_cast<float*>(d.K32), ntens);
     TNMC_CUDA_TRY(cudaGetLastError());
   }
   return TNMC_OK;
@@ -126,14 +130,16 @@ tnmc_status tnmc_launch_derive(tnmc_env* env, int mask, cudaStream_t stream) {
 
 namespace tnmc {
 namespace {
-// transposed FP32 copy [b][a][s] from the left layout [a][s][b]
-__global__ void rederive_f32_kernel(const float* L, float* R, int P, size_t ntens) {
+// FP32 copies [b][a][s] and [a][b][s] from the left layout [a][s][b]
+__global__ void rederive_f32_kernel(const float* L, float* R, float* K, int P, size_t ntens) {
   const size_t per = (size_t)P * 2 * P;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < ntens * per; i += (size_t)gridDim.x * blockDim.x) {
     const size_t t = i / per;
     const int rem = (int)(i % per);
     const int b = rem % P, s = (rem / P) & 1, aa = rem / (2 * P);
-    R[t * per + ((size_t)b * P + aa) * 2 + s] = L[i];
+    const float v = L[i];
+    R[t * per + ((size_t)b * P + aa) * 2 + s] = v;
+    K[t * per + ((size_t)aa * P + b) * 2 + s] = v;
   }
 }
 }  // namespace
@@ -142,7 +148,8 @@ __global__ void rederive_f32_kernel(const float* L, float* R, int P, size_t nten
 tnmc_status tnmc_launch_rederive_f32(tnmc_env* env, cudaStream_t stream) {
   using namespace tnmc;
   DeviceEnv& d = env->d;
-  rederive_f32_kernel<<<1024, 256, 0, stream>>>(d.L32, const_cast<float*>(d.R32), d.P, (size_t)d.Lx * d.Ly);
+  rederive_f32_kernel<<<1024, 256, 0, stream>>>(d.L32, const_cast<float*>(d.R32), const_cast<float*>(d.K32), d.P,
+                                                (size_t)d.Lx * d.Ly);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }
@@ -153,20 +160,25 @@ tnmc_status tnmc_launch_sample(const tnmc_env* env, int precision, int64_t B, ui
   using namespace tnmc;
   const DeviceEnv& d = env->d;
   if (B == 0) return TNMC_OK;
-  if (precision == TNMC_F64)
-    return launch_sample_t<double, 64>(env, d.M64, d.R64, d.fe, B, seed, offset, spins_in, spins_out, logq,
-                                       energy, flags, stream);
+  int dev = 0, nsm = 0, max_smem = 0;
+  TNMC_CUDA_TRY(cudaGetDevice(&dev));
+  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  if (precision == TNMC_F64) {
+    const SampleArgs<double> a{d, d.M64, d.R64, d.fe, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
+    switch (f64_tile_samples(B, d.P, nsm)) {
+      case 32: return launch_sample_f64<8, 4>(env, a, nsm, stream);
+      case 16: return launch_sample_f64<8, 2>(env, a, nsm, stream);
+      case 8: return launch_sample_f64<8, 1>(env, a, nsm, stream);
+      case 4: return launch_sample_f64<4, 1>(env, a, nsm, stream);
+      default: return launch_sample_f64<2, 1>(env, a, nsm, stream);
+    }
+  }
   if (precision == TNMC_F32) {
-    // 128 samples per CTA, or 64 when that leaves SMs without a tile (one thread per sample
-    // either way, so every sample's arithmetic is the same)
-    int dev = 0, nsm = 0;
-    TNMC_CUDA_TRY(cudaGetDevice(&dev));
-    TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    if ((B + 127) / 128 < 2 * (int64_t)nsm)
-      return launch_sample_t<float, 64>(env, d.L32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq,
-                                        energy, flags, stream);
-    return launch_sample_t<float, 128>(env, d.L32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq,
-                                       energy, flags, stream);
+    const SampleArgs<float> a{d, d.K32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
+    return by_f32_block(f32_block(B, d.P, nsm), d.P, [&](auto sb, auto xbm) -> tnmc_status {
+      return launch_sample_f32<decltype(sb)::value, decltype(xbm)::value>(env, a, nsm, max_smem, stream);
+    });
   }
   if (precision == TNMC_BF16)
     return tnmc_launch_sample_tc(env, B, seed, offset, spins_in, spins_out, logq, energy, flags, stream);
