@@ -3,241 +3,630 @@
 // evaluation (Sec. 2, eq. pi-approx; App. A): per-site normalised, clamped
 // conditionals, power-of-two rescalings treated as constants.
 //
-// One thread owns one sample, a CTA owns 128 samples.  Per row r:
+// Per row r and sample:
 //   1. forward right sweep  R_c = k'_c sum_s f_c(s) M_c[s] R_{c+1}      (stack)
 //   2. forward left sweep   Lambda_{c+1} = k_c f_c(s_c) Lambda_c M_c[s_c]   (stack),
 //      raw weights w_c(s) = f_c(s) <Lambda_c M_c[s], R_{c+1}>
-//   3. g_c(s) = d/dw_c(s) [w log w_c(s_c) - w log(w_+ + w_-)], zero where clamped
-//   4. right-to-left adjoint of Lambda:
-//        Lbar_c = sum_s g_c(s) M_c[s] R_{c+1} + k_c f_c(s_c) M_c[s_c] Lbar_{c+1}
+//   3. g_c(s) = d/dw_c(s) [w log w_c(s_c) - w log(w_+ + w_-)] f_c(s), zero where clamped
+//   4. right-to-left adjoint of Lambda (stack):
+//        Lbar_c = sum_s M_c[s] Y_s,  Y_s = g_c(s) R_{c+1} + [s = s_c] k_c f_c(s) Lbar_{c+1}
 //   5. left-to-right adjoint of R and the gradient of site c:
-//        Rbar_{c+1} = sum_s g_c(s) (Lambda_c M_c[s]) + k'_c sum_s f_c(s) M_c[s]^T Rbar_c
-//        G_c[a,s,b] += sum_t Lambda_c[a] Y_s[b] + Rbar_c[a] Z_s[b]
-//          Y_s = g_c(s) R_{c+1} + [s = s_c] k_c f_c(s) Lbar_{c+1},  Z_s = k'_c f_c(s) R_{c+1}
-//      The sum over the CTA's samples is a small (P x 2*128) . (2*128 x P) contraction
-//      per site done in shared memory; each CTA adds its partial with one atomic per
-//      element.
+//        Rbar_{c+1} = sum_s M_c[s]^T V_s,  V_s = g_c(s) Lambda_c + k'_c f_c(s) Rbar_c
+//        G_c[a,s,b] += sum_t V_s[a] R_{c+1}[b] + W_s[a] Lbar_{c+1}[b],
+//          W_s = [s = s_c] k_c f_c(s) Lambda_c
+//
+// A CTA of 4 warps owns 32 samples.  Its 128 threads are 8 sample lanes (4 samples each) x 16
+// output lanes, so every sweep is a register-blocked product whose operands come from shared
+// memory (vectors, and site tensors through a cp.async ring); the site gradient is a
+// (2 chi x 32) . (32 x chi) product over the CTA's samples with up to 8 x 8 outputs per thread,
+// added to global memory by vector reductions.  One __syncthreads per site and sweep: vectors
+// ping-pong between two buffer sets, and a sample's rescaling uses the previous vector's
+// largest entry.  The stacks are read back by the threads that wrote them.
+//
+// What bounds it: shared-memory words (8 per 16 FMAs in the sweeps at chi = 32) and, for
+// batches of a few thousand samples, the barrier and load latencies of 2 CTAs per SM.  One
+// thread per sample without register blocks took 67 ms for 12 x 48, chi = 32, 8192 samples;
+// this form takes 5.3 ms (11.6 TFLOP/s).
 #include <math.h>
 
 #include "common.cuh"
+#include "sample_f32_kernel.cuh"
 
 namespace tnmc {
 namespace {
 
-// NT samples per CTA (one per thread); vectors live in shared memory with stride NT + 1
-// (conflict free).  128 up to P = 52 for large batches; 64 above P = 52 (so that P = 64 fits
-// the shared memory) and for batches too small to give every SM two 128-sample tiles.
+constexpr int kGT = 32;              // samples per CTA
+constexpr int kGThreads = 128;
+constexpr int kGStride = kGT + 4;    // floats per vector row (16 B aligned, rows 4 banks apart)
 
 struct GradArgs {
   DeviceEnv e;
-  const float* L;       // [Ly][Lx][P][2][P]
-  const float* Rt;      // [Ly][Lx][P][P][2]
+  const float* K;       // [Ly][Lx][P][P][2]  [a][b][s]
+  const float* Rt;      // [Ly][Lx][P][P][2]  [b][a][s]
   const float* fe;      // [Ly][Lx][2]
   int64_t B;
   const int8_t* spins;
   const float* weights;
   float* grad;          // [Ly][Lx][P][2][P], accumulated
-  float* scratch;       // per CTA: 3 stacks [Lx+1][P][NT] + 4 x [Lx][NT]
+  float* scratch;       // per CTA: grad_cta_floats
 };
 
-__device__ inline float scale2f(float x, int e) { return scalbnf(x, e); }
+// Per CTA: three stacks [Lx + 1][P][kGT] (R, Lambda, Lbar) and per site and sample w / g of
+// both spins and the exponents of k, k'.
+inline __host__ __device__ size_t grad_cta_floats(int P, int Lx) {
+  return (size_t)3 * (Lx + 1) * P * kGT + (size_t)4 * Lx * kGT;
+}
 
-template <int kNT>
-__global__ void __launch_bounds__(kNT) logq_grad_kernel(GradArgs a) {
-  constexpr int kSP = kNT + 1;
-  extern __shared__ float sm[];
+// Shared memory: the tensor ring, two buffer sets of 6 P vector rows, partial maxima and
+// weights, field factors, bond dimensions and spin masks of the row, sample flags.
+struct GradSmem {
+  int nbuf;
+  size_t set, mpart, wpart, fer, bond, mask, ok, total;
+};
+inline __host__ __device__ GradSmem grad_smem(int P, int Lx) {
+  GradSmem m;
+  m.nbuf = P > 32 ? 2 : 3;
+  size_t o = ((size_t)m.nbuf * P * 2 * P + 128) * sizeof(float);
+  m.set = o;
+  o += (size_t)2 * 6 * P * kGStride * sizeof(float);
+  m.mpart = o;
+  o += (size_t)2 * 4 * kGT * sizeof(float);
+  m.wpart = o;
+  o += (size_t)2 * 4 * 2 * kGT * sizeof(float);
+  m.fer = o;
+  o += (size_t)2 * Lx * sizeof(float);
+  m.bond = o;
+  o += (size_t)(Lx + 1) * sizeof(int);
+  m.mask = o;
+  o += (size_t)2 * Lx * sizeof(uint32_t);
+  m.ok = o;
+  o += kGT * sizeof(int);
+  m.total = o;
+  return m;
+}
+
+// f(IntF<XB>): outputs per thread for dX outputs on 16 output lanes
+template <class F>
+__device__ __forceinline__ void by_outputs(int dX, F&& f) {
+  if (dX <= 16) f(IntF<1>{});
+  else if (dX <= 32) f(IntF<2>{});
+  else if (dX <= 48) f(IntF<3>{});
+  else f(IntF<4>{});
+}
+
+__device__ __forceinline__ void load4(const float* p, float (&v)[4]) { load_run<4>(p, v); }
+
+// acc[s][j][b] = sum_k M[k][x0 + j][s] X[k][b]  (x0 = XB ol)
+template <int XB>
+__device__ __forceinline__ void contract_out(const float* M, int P, int dK, const float* X, int ol, int sl,
+                                             float (&acc)[2][XB][4]) {
+#pragma unroll
+  for (int j = 0; j < XB; ++j)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[0][j][b] = acc[1][j][b] = 0.0f;
+  const float* m = M + 2 * XB * ol;
+  const float* x = X + 4 * sl;
+#pragma unroll 4
+  for (int k = 0; k < dK; ++k) {
+    float xv[4], mv[2 * XB];
+    load4(x + k * kGStride, xv);
+    load_run<2 * XB>(m + (size_t)k * 2 * P, mv);
+#pragma unroll
+    for (int j = 0; j < XB; ++j)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        acc[0][j][b] = fmaf(mv[2 * j], xv[b], acc[0][j][b]);
+        acc[1][j][b] = fmaf(mv[2 * j + 1], xv[b], acc[1][j][b]);
+      }
+  }
+}
+
+// acc[j][b] = sum_k sum_s M[k][x0 + j][s] Y[2 k + s][b]
+template <int XB>
+__device__ __forceinline__ void contract_in(const float* M, int P, int dK, const float* Y, int ol, int sl,
+                                            float (&acc)[XB][4]) {
+#pragma unroll
+  for (int j = 0; j < XB; ++j)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[j][b] = 0.0f;
+  const float* m = M + 2 * XB * ol;
+  const float* y = Y + 4 * sl;
+#pragma unroll 4
+  for (int k = 0; k < dK; ++k) {
+    float y0[4], y1[4], mv[2 * XB];
+    load4(y + (2 * k) * kGStride, y0);
+    load4(y + (2 * k + 1) * kGStride, y1);
+    load_run<2 * XB>(m + (size_t)k * 2 * P, mv);
+#pragma unroll
+    for (int j = 0; j < XB; ++j)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        acc[j][b] = fmaf(mv[2 * j], y0[b], acc[j][b]);
+        acc[j][b] = fmaf(mv[2 * j + 1], y1[b], acc[j][b]);
+      }
+  }
+}
+
+// G[rho][b] += sum_t V[rho][t] R[b][t] + W[rho][t] Lb[b][t], rho = 2 a + s < nr, b < nc.  The four
+// warps take 2 x 2 blocks of 8 Q x 4 Q outputs, a thread Q x Q of them.
+template <int Q>
+__device__ __forceinline__ void site_gradient(const float* V, const float* W, const float* R, const float* Lb, int P,
+                                              int nr, int nc, float* G) {
+  const bool vec = (reinterpret_cast<uintptr_t>(G) & 15) == 0;      // the caller's buffer may be only 4-byte aligned
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row0 = (warp & 1) * 8 * Q + (lane & 7), col0 = ((warp >> 1) * 4 + (lane >> 3)) * Q;
+  float acc[Q][Q];
+  int ro[Q], co[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    ro[i] = min(row0 + 8 * i, 2 * P - 1) * kGStride;
+    co[i] = min(col0 + i, P - 1) * kGStride;
+#pragma unroll
+    for (int j = 0; j < Q; ++j) acc[i][j] = 0.0f;
+  }
+  auto add = [&](const float* A, const float* C) {
+#pragma unroll 1
+    for (int t = 0; t < kGT; t += 4) {
+      float av[Q][4], cv[Q][4];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        load4(A + ro[i] + t, av[i]);
+        load4(C + co[i] + t, cv[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int j = 0; j < Q; ++j)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[i][j] = fmaf(av[i][q], cv[j][q], acc[i][j]);
+    }
+  };
+  add(V, R);
+  add(W, Lb);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int rho = row0 + 8 * i;
+    if (rho >= nr) continue;
+    float* g = G + (size_t)rho * P + col0;
+    if constexpr (Q % 4 == 0) {
+#pragma unroll
+      for (int j = 0; j < Q; j += 4) {
+        if (vec && col0 + j + 3 < nc) {
+          atomicAdd(reinterpret_cast<float4*>(g + j), make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]));
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (col0 + j + q < nc) atomicAdd(g + j + q, acc[i][j + q]);
+        }
+      }
+    } else if constexpr (Q % 2 == 0) {
+#pragma unroll
+      for (int j = 0; j < Q; j += 2) {
+        if (vec && col0 + j + 1 < nc) {
+          atomicAdd(reinterpret_cast<float2*>(g + j), make_float2(acc[i][j], acc[i][j + 1]));
+        } else {
+#pragma unroll
+          for (int q = 0; q < 2; ++q)
+            if (col0 + j + q < nc) atomicAdd(g + j + q, acc[i][j + q]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < Q; ++j)
+        if (col0 + j < nc) atomicAdd(g + j, acc[i][j]);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const unsigned kFull = 0xffffffffu;
   const int Lx = a.e.Lx, Ly = a.e.Ly, P = a.e.P;
-  const int W = (Lx + 31) >> 5;
-  const int t = threadIdx.x;
-  float* V0 = sm;                        // [P][SP]  Lambda_c (P1)
-  float* V2 = V0 + P * kSP;              // [P][SP]  Rbar_c (P2)
-  float* V3 = V2 + P * kSP;              // [P][SP]  scratch vector
-  float* Y = V3 + P * kSP;               // [2][P][SP]
-  float* Z = Y + 2 * P * kSP;            // [2][P][SP]
-  uint32_t* bits_prev = reinterpret_cast<uint32_t*>(Z + 2 * P * kSP);   // [W][NT]
-  uint32_t* bits_cur = bits_prev + W * kNT;
-  const int64_t tile = blockIdx.x;
-  const int64_t b = tile * kNT + t;
-  const bool active = b < a.B;
-  const int n = Lx * Ly;
-  const size_t stack = (size_t)(Lx + 1) * P * kNT;
-  float* Rs = a.scratch + (size_t)blockIdx.x * (3 * stack + 4 * (size_t)Lx * kNT);
-  float* Ls = Rs + stack;
-  float* LBs = Ls + stack;
-  float* w0s = LBs + stack;              // [Lx][NT] raw w(-)
-  float* w1s = w0s + (size_t)Lx * kNT;   // [Lx][NT] raw w(+)
-  int* ek = reinterpret_cast<int*>(w1s + (size_t)Lx * kNT);    // exponent of k_c (Lambda_{c+1})
-  int* ekp = ek + (size_t)Lx * kNT;                           // exponent of k'_c (R_c)
-  const float wt = active ? a.weights[b] : 0.0f;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sl = lane & 7, ol = (lane >> 3) + 4 * warp;      // samples 4 sl .. 4 sl + 3, outputs XB ol ..
+  const GradSmem lay = grad_smem(P, Lx);
+  float* ring = reinterpret_cast<float*>(smem_raw);
+  float* set0 = reinterpret_cast<float*>(smem_raw + lay.set);
+  const size_t set_sz = (size_t)6 * P * kGStride;
+  float* mpart = reinterpret_cast<float*>(smem_raw + lay.mpart);     // [2][4][kGT]
+  float* wpart = reinterpret_cast<float*>(smem_raw + lay.wpart);     // [2][4][2][kGT]
+  float* fer = reinterpret_cast<float*>(smem_raw + lay.fer);
+  int* bond = reinterpret_cast<int*>(smem_raw + lay.bond);
+  uint32_t* prev = reinterpret_cast<uint32_t*>(smem_raw + lay.mask);
+  uint32_t* cur = prev + Lx;
+  int* okf = reinterpret_cast<int*>(smem_raw + lay.ok);
+  const size_t n = (size_t)Lx * Ly, tstride = (size_t)P * 2 * P, slot = (size_t)P * kGT;
+  float* Rs = a.scratch + (size_t)blockIdx.x * grad_cta_floats(P, Lx);
+  float* Ls = Rs + (Lx + 1) * slot;
+  float* Bs = Ls + (Lx + 1) * slot;
+  float* w0s = Bs + (Lx + 1) * slot;             // [Lx][kGT]: raw w(-), then g(-)
+  float* w1s = w0s + (size_t)Lx * kGT;
+  int* ek = reinterpret_cast<int*>(w1s + (size_t)Lx * kGT);      // exponent of k_c
+  int* ekp = ek + (size_t)Lx * kGT;                               // exponent of k'_c
 
-  for (int wd = 0; wd < W; ++wd) bits_prev[wd * kNT + t] = 0u;
-  for (int r = 0; r < Ly; ++r) {
-    const int32_t* bond = a.e.bond + r * (Lx + 1);
-    const float* fer = a.fe + (size_t)r * Lx * 2;
-    for (int wd = 0; wd < W; ++wd) bits_cur[wd * kNT + t] = 0u;
-    if (active) {
-      const int8_t* src = a.spins + (size_t)b * n + (size_t)r * Lx;
-      for (int c = 0; c < Lx; ++c)
-        if (src[c] > 0) bits_cur[(c >> 5) * kNT + t] |= 1u << (c & 31);
-    }
-    auto fval = [&](int c, int s) -> float {
-      if (r == 0) return 1.0f;
-      const bool up = (bits_prev[(c >> 5) * kNT + t] >> (c & 31)) & 1u;
-      return ((up ? 1 : 0) == s) ? fer[2 * c + 1] : fer[2 * c];
+  const int nstep = 4 * Lx - 3, dist = lay.nbuf - 1;
+  for (int64_t base = (int64_t)blockIdx.x * kGT; base < a.B; base += (int64_t)gridDim.x * kGT) {
+    const int rows = (a.B - base) < kGT ? (int)(a.B - base) : kGT;
+    __syncthreads();       // the previous tile is done with shared memory
+    for (int c = tid; c < Lx; c += kGThreads) prev[c] = 0u;
+    int pr = 0, pi = 0, pbuf = 0;
+    auto copy_next = [&]() {
+      if (pr < Ly) {
+        // steps: right sweep, left sweep, Lambda adjoint, R adjoint (sites 0 .. Lx - 2)
+        const int p1 = Lx - 1, p2 = p1 + Lx, p3 = p2 + Lx - 1;
+        const int c = pi < p1 ? Lx - 1 - pi : pi < p2 ? pi - p1 : pi < p3 ? Lx - 1 - (pi - p2) : pi - p3;
+        const bool right = pi < p1 || (pi >= p2 && pi < p3);
+        const float* src = (right ? a.Rt : a.K) + ((size_t)pr * Lx + c) * tstride;
+        float* dst = ring + (size_t)pbuf * tstride;
+        for (int q = tid; q < P * P / 2; q += kGThreads) cp_async16(dst + 4 * q, src + 4 * q);
+        if (++pi == nstep) {
+          pi = 0;
+          ++pr;
+        }
+      }
+      if (++pbuf == lay.nbuf) pbuf = 0;
+      cp_async_commit();
     };
-    auto spin = [&](int c) -> int { return (bits_cur[(c >> 5) * kNT + t] >> (c & 31)) & 1u; };
-    // ---- 1. right sweep ----
-    for (int k = 0; k < P; ++k) Rs[((size_t)Lx * P + k) * kNT + t] = (k == 0) ? 1.0f : 0.0f;
-    for (int c = Lx - 1; c >= 1; --c) {
-      const int dc = bond[c], dc1 = bond[c + 1];
-      const float f0 = fval(c, 0), f1 = fval(c, 1);
-      const float* M = a.L + ((size_t)r * Lx + c) * P * 2 * P;
-      const float* Rn = Rs + (size_t)(c + 1) * P * kNT;
-      float mx = 0.0f;
-      for (int aa = 0; aa < dc; ++aa) {
-        float s0 = 0.0f, s1 = 0.0f;
-        for (int bb = 0; bb < dc1; ++bb) {
-          const float rb = Rn[bb * kNT + t];
-          s0 = fmaf(__ldg(M + ((size_t)aa * 2) * P + bb), rb, s0);
-          s1 = fmaf(__ldg(M + ((size_t)aa * 2 + 1) * P + bb), rb, s1);
-        }
-        const float v = f0 * s0 + f1 * s1;
-        V3[aa * kSP + t] = v;
-        mx = fmaxf(mx, fabsf(v));
-      }
-      const int e = (mx > 0.0f) ? -ilogbf(mx) : 0;
-      ekp[(size_t)c * kNT + t] = e;
-      float* Rc = Rs + (size_t)c * P * kNT;
-      for (int aa = 0; aa < P; ++aa) Rc[aa * kNT + t] = (aa < dc) ? scale2f(V3[aa * kSP + t], e) : 0.0f;
-    }
-    // ---- 2. left sweep (forced) ----
-    for (int k = 0; k < P; ++k) Ls[(size_t)k * kNT + t] = (k == 0) ? 1.0f : 0.0f;
-    for (int c = 0; c < Lx; ++c) {
-      const int dc = bond[c], dc1 = bond[c + 1];
-      const float f0 = fval(c, 0), f1 = fval(c, 1);
-      const int s = spin(c);
-      const float* M = a.L + ((size_t)r * Lx + c) * P * 2 * P;
-      const float* Lc = Ls + (size_t)c * P * kNT;
-      const float* Rn = Rs + (size_t)(c + 1) * P * kNT;
-      float w0 = 0.0f, w1 = 0.0f, mx = 0.0f;
-      for (int bb = 0; bb < dc1; ++bb) {
-        float u0 = 0.0f, u1 = 0.0f;
-        for (int aa = 0; aa < dc; ++aa) {
-          const float la = Lc[aa * kNT + t];
-          u0 = fmaf(la, __ldg(M + ((size_t)aa * 2) * P + bb), u0);
-          u1 = fmaf(la, __ldg(M + ((size_t)aa * 2 + 1) * P + bb), u1);
-        }
-        const float rb = Rn[bb * kNT + t];
-        w0 = fmaf(u0, rb, w0);
-        w1 = fmaf(u1, rb, w1);
-        const float us = (s ? u1 : u0) * (s ? f1 : f0);
-        V3[bb * kSP + t] = us;
-        mx = fmaxf(mx, fabsf(us));
-      }
-      w0s[(size_t)c * kNT + t] = w0 * f0;
-      w1s[(size_t)c * kNT + t] = w1 * f1;
-      const int e = (mx > 0.0f) ? -ilogbf(mx) : 0;
-      ek[(size_t)c * kNT + t] = e;
-      float* Ln = Ls + (size_t)(c + 1) * P * kNT;
-      for (int bb = 0; bb < P; ++bb) Ln[bb * kNT + t] = (bb < dc1) ? scale2f(V3[bb * kSP + t], e) : 0.0f;
-    }
-    // per-site weight adjoints g_c(s); a sample with a non-positive normaliser, or with
-    // q = 0, contributes nothing (its log q is not differentiable)
-    bool ok = wt != 0.0f;
-    for (int c = 0; c < Lx && ok; ++c) {
-      const float w0 = fmaxf(w0s[(size_t)c * kNT + t], 0.0f), w1 = fmaxf(w1s[(size_t)c * kNT + t], 0.0f);
-      const float ws = spin(c) ? w1 : w0;
-      ok = (w0 + w1 > 0.0f) && isfinite(w0 + w1) && ws > 0.0f;
-    }
-    auto gw = [&](int c, int s_) -> float {
-      if (!ok) return 0.0f;
-      const float w0r = w0s[(size_t)c * kNT + t], w1r = w1s[(size_t)c * kNT + t];
-      const float w0 = fmaxf(w0r, 0.0f), w1 = fmaxf(w1r, 0.0f);
-      const int sc = spin(c);
-      const float ws = sc ? w1 : w0;
-      float g = -1.0f / (w0 + w1);
-      if (s_ == sc) g += 1.0f / ws;
-      const float raw = s_ ? w1r : w0r;
-      return (raw > 0.0f) ? wt * g * fval(c, s_) : 0.0f;
+    for (int q = 0; q < dist; ++q) copy_next();
+    int buf = 0;
+    auto begin_step = [&]() -> const float* {
+      if (dist == 2) cp_async_wait<1>();
+      else cp_async_wait<0>();
+      __syncthreads();
+      copy_next();
+      const float* M = ring + (size_t)buf * tstride;
+      if (++buf == lay.nbuf) buf = 0;
+      return M;
     };
-    // ---- 4. Lambda adjoint, right to left: LBs[c] = Lbar_c (c = 1..Lx) ----
-    for (int k = 0; k < P; ++k) LBs[((size_t)Lx * P + k) * kNT + t] = 0.0f;
-    for (int c = Lx - 1; c >= 1; --c) {
-      const int dc = bond[c], dc1 = bond[c + 1];
-      const int s = spin(c);
-      const float g0 = gw(c, 0), g1 = gw(c, 1);
-      const float kf = scale2f(1.0f, ek[(size_t)c * kNT + t]) * fval(c, s);
-      const float* M = a.L + ((size_t)r * Lx + c) * P * 2 * P;
-      const float* Rn = Rs + (size_t)(c + 1) * P * kNT;
-      const float* LBn = LBs + (size_t)(c + 1) * P * kNT;
-      float* LBc = LBs + (size_t)c * P * kNT;
-      for (int aa = 0; aa < P; ++aa) {
-        float acc = 0.0f;
-        if (aa < dc) {
-          for (int bb = 0; bb < dc1; ++bb) {
-            const float m0 = __ldg(M + ((size_t)aa * 2) * P + bb), m1 = __ldg(M + ((size_t)aa * 2 + 1) * P + bb);
-            const float rb = Rn[bb * kNT + t];
-            acc = fmaf(g0 * m0 + g1 * m1, rb, acc);
-            acc = fmaf(kf * (s ? m1 : m0), LBn[bb * kNT + t], acc);
+    // the rescaling exponent of this thread's samples from the previous vector's maxima
+    auto lag = [&](int par, int (&e)[4]) {
+      float m[4], q[4];
+      load4(mpart + par * 4 * kGT + 4 * sl, m);
+#pragma unroll
+      for (int w = 1; w < 4; ++w) {
+        load4(mpart + (par * 4 + w) * kGT + 4 * sl, q);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) m[b] = fmaxf(m[b], q[b]);
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b) e[b] = exponent_f32(__float_as_int(m[b]));
+    };
+    auto put_max = [&](int par, float (&m)[4]) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        m[b] = fmaxf(m[b], __shfl_xor_sync(kFull, m[b], 8));
+        m[b] = fmaxf(m[b], __shfl_xor_sync(kFull, m[b], 16));
+      }
+      if (lane < 8) store_run<4>(mpart + (par * 4 + warp) * kGT + 4 * sl, m);
+    };
+    auto put_one = [&](float* X) {       // the boundary vector: one row of ones
+      if (tid < kGT) X[tid] = 1.0f;
+      if (tid < 4 * kGT) mpart[tid] = 1.0f;      // parity 0
+    };
+
+    for (int r = 0; r < Ly; ++r) {
+      __syncthreads();
+      for (int c = tid; c <= Lx; c += kGThreads) bond[c] = a.e.bond[r * (Lx + 1) + c];
+      for (int c = tid; c < 2 * Lx; c += kGThreads) fer[c] = r == 0 ? 1.0f : a.fe[(size_t)r * Lx * 2 + c];
+      for (int c = tid; c < Lx; c += kGThreads) {
+        const int8_t* src = a.spins + (size_t)base * n + (size_t)r * Lx + c;
+        uint32_t m = 0;
+#pragma unroll 8
+        for (int s = 0; s < rows; ++s) m |= (src[(size_t)s * n] > 0 ? 1u : 0u) << s;
+        cur[c] = m;
+      }
+      if (tid < kGT) {
+        okf[tid] = 1;
+        Rs[Lx * slot + tid] = 1.0f;      // R_Lx, Lambda_0 = 1 and Lbar_Lx = 0 (one bond)
+        Ls[tid] = 1.0f;
+        Bs[Lx * slot + tid] = 0.0f;
+      }
+      put_one(set0);
+      // ---- 1. right sweep ----
+      int step = 0;
+      for (int c = Lx - 1; c >= 1; --c, ++step) {
+        const float* M = begin_step();
+        const int dK = bond[c + 1], dX = bond[c];
+        const uint32_t up = prev[c];
+        const float fdiff = fer[2 * c], fsame = fer[2 * c + 1];
+        const float* X = set0 + (step & 1) * set_sz;
+        float* Xn = set0 + ((step + 1) & 1) * set_sz;
+        by_outputs(dX, [&](auto xbc) {
+          constexpr int XB = decltype(xbc)::value;
+          float acc[2][XB][4], m[4];
+          int e[4];
+          contract_out<XB>(M, P, dK, X, ol, sl, acc);
+          lag(step & 1, e);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const bool u = (up >> (4 * sl + b)) & 1u;
+            const float sc = pow2_f32(-e[b]);
+            const float f0 = (u ? fdiff : fsame) * sc, f1 = (u ? fsame : fdiff) * sc;
+            m[b] = 0.0f;
+#pragma unroll
+            for (int j = 0; j < XB; ++j) {
+              acc[0][j][b] = fmaf(f0, acc[0][j][b], f1 * acc[1][j][b]);
+              if (XB * ol + j < dX) m[b] = fmaxf(m[b], fabsf(acc[0][j][b]));
+            }
           }
-        }
-        LBc[aa * kNT + t] = acc;
-      }
-    }
-    // ---- 5. R adjoint left to right, and the site gradients ----
-    for (int k = 0; k < P; ++k) V2[k * kSP + t] = 0.0f;   // Rbar_0 (unused: R_0 is never formed)
-    for (int c = 0; c < Lx; ++c) {
-      const int dc = bond[c], dc1 = bond[c + 1];
-      const int s = spin(c);
-      const float f0 = fval(c, 0), f1 = fval(c, 1);
-      const float g0 = gw(c, 0), g1 = gw(c, 1);
-      const float kf = scale2f(1.0f, ek[(size_t)c * kNT + t]) * (s ? f1 : f0);
-      const float kp = (c >= 1) ? scale2f(1.0f, ekp[(size_t)c * kNT + t]) : 0.0f;
-      const float* M = a.L + ((size_t)r * Lx + c) * P * 2 * P;
-      const float* Lc = Ls + (size_t)c * P * kNT;
-      const float* Rn = Rs + (size_t)(c + 1) * P * kNT;
-      const float* LBn = LBs + (size_t)(c + 1) * P * kNT;
-      // operands of G_c: P1 = Lambda_c, P2 = Rbar_c, Y_s, Z_s
-      for (int k = 0; k < P; ++k) {
-        V0[k * kSP + t] = Lc[k * kNT + t];
-        const float rb = Rn[k * kNT + t];
-        const float lb = (c + 1 < Lx) ? LBn[k * kNT + t] : 0.0f;
-        Y[(0 * P + k) * kSP + t] = g0 * rb + (s == 0 ? kf * lb : 0.0f);
-        Y[(1 * P + k) * kSP + t] = g1 * rb + (s == 1 ? kf * lb : 0.0f);
-        Z[(0 * P + k) * kSP + t] = kp * f0 * rb;
-        Z[(1 * P + k) * kSP + t] = kp * f1 * rb;
-      }
-      __syncthreads();
-      // G_c partial over the CTA's samples: thread -> (a, s, b) entries
-      float* G = a.grad + ((size_t)r * Lx + c) * P * 2 * P;
-      for (int idx = t; idx < dc * 2 * dc1; idx += kNT) {
-        const int bb = idx % dc1, s_ = (idx / dc1) & 1, aa = idx / (2 * dc1);
-        const float* y = Y + (size_t)(s_ * P + bb) * kSP;
-        const float* z = Z + (size_t)(s_ * P + bb) * kSP;
-        const float* p1 = V0 + (size_t)aa * kSP;
-        const float* p2 = V2 + (size_t)aa * kSP;
-        float acc = 0.0f;
-        for (int q = 0; q < kNT; ++q) acc = fmaf(p1[q], y[q], fmaf(p2[q], z[q], acc));
-        if (acc != 0.0f) atomicAdd(G + ((size_t)aa * 2 + s_) * P + bb, acc);
-      }
-      __syncthreads();
-      // Rbar_{c+1} = sum_s g(s) Lambda_c M_c[s] + k'_c sum_s f(s) M_c[s]^T Rbar_c
-      if (c + 1 < Lx) {
-        for (int bb = 0; bb < dc1; ++bb) {
-          float acc = 0.0f;
-          for (int aa = 0; aa < dc; ++aa) {
-            const float m0 = __ldg(M + ((size_t)aa * 2) * P + bb), m1 = __ldg(M + ((size_t)aa * 2 + 1) * P + bb);
-            acc = fmaf(Lc[aa * kNT + t], g0 * m0 + g1 * m1, acc);
-            acc = fmaf(V2[aa * kSP + t], kp * (f0 * m0 + f1 * m1), acc);
+#pragma unroll
+          for (int j = 0; j < XB; ++j) {
+            const int x = XB * ol + j;
+            if (x < dX) {
+              store_run<4>(Xn + x * kGStride + 4 * sl, acc[0][j]);
+              store_run<4>(Rs + c * slot + x * kGT + 4 * sl, acc[0][j]);
+            }
           }
-          V3[bb * kSP + t] = acc;
+          if (ol == 0) *reinterpret_cast<int4*>(ekp + c * kGT + 4 * sl) = make_int4(-e[0], -e[1], -e[2], -e[3]);
+          put_max((step + 1) & 1, m);
+        });
+      }
+      // ---- 2. left sweep (forced) ----
+      __syncthreads();
+      put_one(set0);
+      step = 0;
+      auto finish_weights = [&](int c) {      // raw weights of site c from the four warps' sums
+        if (tid < 2 * kGT) {
+          const int s = tid / kGT, t = tid % kGT;
+          const float* wp = wpart + (c & 1) * 8 * kGT + s * kGT + t;
+          const float w = (wp[0] + wp[2 * kGT]) + (wp[4 * kGT] + wp[6 * kGT]);
+          const bool same = (int)((prev[c] >> t) & 1u) == s;
+          (s ? w1s : w0s)[c * kGT + t] = w * (same ? fer[2 * c + 1] : fer[2 * c]);
         }
-        __syncthreads();
-        for (int k = 0; k < P; ++k) V2[k * kSP + t] = (k < dc1) ? V3[k * kSP + t] : 0.0f;
+      };
+      for (int c = 0; c < Lx; ++c, ++step) {
+        const float* M = begin_step();
+        if (c > 0) finish_weights(c - 1);
+        const int dK = bond[c], dX = bond[c + 1];
+        const uint32_t up = prev[c], sp = cur[c];
+        const float fdiff = fer[2 * c], fsame = fer[2 * c + 1];
+        const float* X = set0 + (step & 1) * set_sz;
+        float* Xn = set0 + ((step + 1) & 1) * set_sz;
+        by_outputs(dX, [&](auto xbc) {
+          constexpr int XB = decltype(xbc)::value;
+          float rv[XB][4];
+#pragma unroll
+          for (int j = 0; j < XB; ++j) {
+            const int x = XB * ol + j;
+            if (x < dX) load4(Rs + (c + 1) * slot + x * kGT + 4 * sl, rv[j]);
+          }
+          float acc[2][XB][4], m[4], w0[4], w1[4];
+          int e[4];
+          contract_out<XB>(M, P, dK, X, ol, sl, acc);
+          lag(step & 1, e);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const bool u = (up >> (4 * sl + b)) & 1u, s = (sp >> (4 * sl + b)) & 1u;
+            const float fs = ((u == s) ? fsame : fdiff) * pow2_f32(-e[b]);
+            m[b] = w0[b] = w1[b] = 0.0f;
+#pragma unroll
+            for (int j = 0; j < XB; ++j) {
+              if (XB * ol + j < dX) {
+                w0[b] = fmaf(acc[0][j][b], rv[j][b], w0[b]);
+                w1[b] = fmaf(acc[1][j][b], rv[j][b], w1[b]);
+                acc[0][j][b] = (s ? acc[1][j][b] : acc[0][j][b]) * fs;
+                m[b] = fmaxf(m[b], fabsf(acc[0][j][b]));
+              }
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < XB; ++j) {
+            const int x = XB * ol + j;
+            if (x < dX) {
+              store_run<4>(Xn + x * kGStride + 4 * sl, acc[0][j]);
+              store_run<4>(Ls + (c + 1) * slot + x * kGT + 4 * sl, acc[0][j]);
+            }
+          }
+          if (ol == 0) *reinterpret_cast<int4*>(ek + c * kGT + 4 * sl) = make_int4(-e[0], -e[1], -e[2], -e[3]);
+          put_max((step + 1) & 1, m);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            w0[b] += __shfl_xor_sync(kFull, w0[b], 8);
+            w1[b] += __shfl_xor_sync(kFull, w1[b], 8);
+            w0[b] += __shfl_xor_sync(kFull, w0[b], 16);
+            w1[b] += __shfl_xor_sync(kFull, w1[b], 16);
+          }
+          if (lane < 8) {
+            store_run<4>(wpart + (c & 1) * 8 * kGT + 2 * warp * kGT + 4 * sl, w0);
+            store_run<4>(wpart + (c & 1) * 8 * kGT + (2 * warp + 1) * kGT + 4 * sl, w1);
+          }
+        });
       }
       __syncthreads();
+      finish_weights(Lx - 1);
+      __syncthreads();
+      // ---- 3. weight adjoints; a sample with a non-positive normaliser, or with q = 0,
+      // contributes nothing (its log q is not differentiable) ----
+      for (int q = tid; q < Lx * kGT; q += kGThreads) {
+        const int c = q / kGT, t = q % kGT;
+        const float w0 = fmaxf(w0s[q], 0.0f), w1 = fmaxf(w1s[q], 0.0f);
+        const float ws = ((cur[c] >> t) & 1u) ? w1 : w0;
+        if (!(w0 + w1 > 0.0f && isfinite(w0 + w1) && ws > 0.0f)) okf[t] = 0;
+      }
+      if (tid < kGT) {
+        const float wt = tid < rows ? a.weights[base + tid] : 0.0f;
+        if (!(wt != 0.0f)) okf[tid] = 0;
+      }
+      __syncthreads();
+      for (int q = tid; q < Lx * kGT; q += kGThreads) {
+        const int c = q / kGT, t = q % kGT;
+        const float w0r = w0s[q], w1r = w1s[q];
+        const float w0 = fmaxf(w0r, 0.0f), w1 = fmaxf(w1r, 0.0f);
+        const bool sc = (cur[c] >> t) & 1u, u = (prev[c] >> t) & 1u;
+        float g0 = 0.0f, g1 = 0.0f;
+        if (okf[t]) {
+          const float wt = a.weights[base + t];
+          const float inv = -1.0f / (w0 + w1), is = 1.0f / (sc ? w1 : w0);
+          if (w0r > 0.0f) g0 = wt * (inv + (sc ? 0.0f : is)) * (u ? fer[2 * c] : fer[2 * c + 1]);
+          if (w1r > 0.0f) g1 = wt * (inv + (sc ? is : 0.0f)) * (u ? fer[2 * c + 1] : fer[2 * c]);
+        }
+        w0s[q] = g0;
+        w1s[q] = g1;
+      }
+      __syncthreads();
+      // this thread's samples that contribute (the others' vectors count as zero below)
+      bool ok[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) ok[b] = okf[4 * sl + b] != 0;
+      // g, k f of the sample's own spin, and the spin, of site c
+      struct SiteW {
+        float g0[4], g1[4], kf[4];
+        uint32_t sp;
+      };
+      auto site_weights = [&](int c, SiteW& w) {
+        load4(w0s + c * kGT + 4 * sl, w.g0);
+        load4(w1s + c * kGT + 4 * sl, w.g1);
+        const int4 e = *reinterpret_cast<const int4*>(ek + c * kGT + 4 * sl);
+        const int ev[4] = {e.x, e.y, e.z, e.w};
+        w.sp = cur[c] >> (4 * sl);
+        const uint32_t up = prev[c] >> (4 * sl);
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          w.kf[b] = ((((up ^ w.sp) >> b) & 1u) ? fer[2 * c] : fer[2 * c + 1]) * pow2_f32(ev[b]);
+      };
+      // Y rows x of site c from R_{c+1} and Lbar_{c+1}
+      auto put_y = [&](float* Y, int x, const float (&rv)[4], const float (&lb)[4], const SiteW& w) {
+        float y0[4], y1[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float rr = ok[b] ? rv[b] : 0.0f, t = w.kf[b] * lb[b];
+          const bool s = (w.sp >> b) & 1u;
+          y0[b] = fmaf(w.g0[b], rr, s ? 0.0f : t);
+          y1[b] = fmaf(w.g1[b], rr, s ? t : 0.0f);
+        }
+        store_run<4>(Y + (2 * x) * kGStride + 4 * sl, y0);
+        store_run<4>(Y + (2 * x + 1) * kGStride + 4 * sl, y1);
+      };
+      // ---- 4. Lambda adjoint, right to left ----
+      if (Lx > 1 && ol == 0) {
+        SiteW w;
+        site_weights(Lx - 1, w);
+        const float one[4] = {1.0f, 1.0f, 1.0f, 1.0f}, zero[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        put_y(set0, 0, one, zero, w);
+      }
+      step = 0;
+      for (int c = Lx - 1; c >= 1; --c, ++step) {
+        const float* M = begin_step();
+        const int dK = bond[c + 1], dX = bond[c];
+        const float* Y = set0 + (step & 1) * set_sz;
+        float* Yn = set0 + ((step + 1) & 1) * set_sz;
+        SiteW w;
+        if (c > 1) site_weights(c - 1, w);
+        by_outputs(dX, [&](auto xbc) {
+          constexpr int XB = decltype(xbc)::value;
+          float rv[XB][4];
+#pragma unroll
+          for (int j = 0; j < XB; ++j) {
+            const int x = XB * ol + j;
+            if (x < dX && c > 1) load4(Rs + c * slot + x * kGT + 4 * sl, rv[j]);
+          }
+          float acc[XB][4];
+          contract_in<XB>(M, P, dK, Y, ol, sl, acc);
+#pragma unroll
+          for (int j = 0; j < XB; ++j) {
+            const int x = XB * ol + j;
+            if (x < dX) {
+              store_run<4>(Bs + c * slot + x * kGT + 4 * sl, acc[j]);
+              if (c > 1) put_y(Yn, x, rv[j], acc[j], w);
+            }
+          }
+        });
+      }
+      __syncthreads();
+      // ---- 5. R adjoint left to right, and the site gradients.  Buffer set: V [2 P], W [2 P],
+      // R [P], Lbar [P] rows of site c ----
+      const int oW = 2 * P * kGStride, oR = 4 * P * kGStride, oL = 5 * P * kGStride;
+      // V and W rows x of site c from Lambda_c and k'_c f Rbar_c (rb holds Rbar_c)
+      auto put_v = [&](float* S, int x, const float (&lv)[4], const float (&rb)[4], const SiteW& w, int c) {
+        const uint32_t up = prev[c] >> (4 * sl);
+        const int4 e = c > 0 ? *reinterpret_cast<const int4*>(ekp + c * kGT + 4 * sl) : make_int4(0, 0, 0, 0);
+        const int ev[4] = {e.x, e.y, e.z, e.w};
+        float v0[4], v1[4], x0[4], x1[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float l = ok[b] ? lv[b] : 0.0f;
+          const float kr = pow2_f32(ev[b]) * rb[b];
+          const bool u = (up >> b) & 1u, s = (w.sp >> b) & 1u;
+          v0[b] = fmaf(w.g0[b], l, (u ? fer[2 * c] : fer[2 * c + 1]) * kr);
+          v1[b] = fmaf(w.g1[b], l, (u ? fer[2 * c + 1] : fer[2 * c]) * kr);
+          const float t = w.kf[b] * l;
+          x0[b] = s ? 0.0f : t;
+          x1[b] = s ? t : 0.0f;
+        }
+        store_run<4>(S + (2 * x) * kGStride + 4 * sl, v0);
+        store_run<4>(S + (2 * x + 1) * kGStride + 4 * sl, v1);
+        store_run<4>(S + oW + (2 * x) * kGStride + 4 * sl, x0);
+        store_run<4>(S + oW + (2 * x + 1) * kGStride + 4 * sl, x1);
+      };
+      // R_{c+1} and Lbar_{c+1} rows of site c
+      auto put_right = [&](float* S, int c) {
+        const int d = bond[c + 1];
+        by_outputs(d, [&](auto xbc) {
+          constexpr int XB = decltype(xbc)::value;
+#pragma unroll
+          for (int j = 0; j < XB; ++j) {
+            const int x = XB * ol + j;
+            if (x < d) {
+              float rv[4], lb[4];
+              load4(Rs + (c + 1) * slot + x * kGT + 4 * sl, rv);
+              load4(Bs + (c + 1) * slot + x * kGT + 4 * sl, lb);
+#pragma unroll
+              for (int b = 0; b < 4; ++b) {
+                rv[b] = ok[b] ? rv[b] : 0.0f;
+                lb[b] = ok[b] ? lb[b] : 0.0f;
+              }
+              store_run<4>(S + oR + x * kGStride + 4 * sl, rv);
+              store_run<4>(S + oL + x * kGStride + 4 * sl, lb);
+            }
+          }
+        });
+      };
+      if (ol == 0) {
+        SiteW w;
+        site_weights(0, w);
+        const float one[4] = {1.0f, 1.0f, 1.0f, 1.0f}, zero[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        put_v(set0, 0, one, zero, w, 0);
+      }
+      put_right(set0, 0);
+      for (int c = 0; c < Lx; ++c) {
+        float* S = set0 + (c & 1) * set_sz;
+        float* Sn = set0 + ((c + 1) & 1) * set_sz;
+        const int dl = bond[c], dr = bond[c + 1];
+        if (c + 1 < Lx) {
+          const float* M = begin_step();
+          SiteW w;
+          site_weights(c + 1, w);
+          by_outputs(dr, [&](auto xbc) {
+            constexpr int XB = decltype(xbc)::value;
+            float lv[XB][4];
+#pragma unroll
+            for (int j = 0; j < XB; ++j) {
+              const int x = XB * ol + j;
+              if (x < dr) load4(Ls + (c + 1) * slot + x * kGT + 4 * sl, lv[j]);
+            }
+            float acc[XB][4];
+            contract_in<XB>(M, P, dl, S, ol, sl, acc);
+#pragma unroll
+            for (int j = 0; j < XB; ++j) {
+              const int x = XB * ol + j;
+              if (x < dr) put_v(Sn, x, lv[j], acc[j], w, c + 1);
+            }
+          });
+          put_right(Sn, c + 1);
+        } else {
+          __syncthreads();
+        }
+        float* G = a.grad + ((size_t)r * Lx + c) * tstride;
+        const int q = (max(dl, dr) + 7) >> 3;
+        if (q <= 1) site_gradient<1>(S, S + oW, S + oR, S + oL, P, 2 * dl, dr, G);
+        else if (q == 2) site_gradient<2>(S, S + oW, S + oR, S + oL, P, 2 * dl, dr, G);
+        else if (q <= 4) site_gradient<4>(S, S + oW, S + oR, S + oL, P, 2 * dl, dr, G);
+        else site_gradient<8>(S, S + oW, S + oR, S + oL, P, 2 * dl, dr, G);
+      }
+      __syncthreads();
+      for (int c = tid; c < Lx; c += kGThreads) prev[c] = cur[c];
     }
-    for (int wd = 0; wd < W; ++wd) bits_prev[wd * kNT + t] = bits_cur[wd * kNT + t];
+    cp_async_wait<0>();
   }
 }
 
@@ -251,37 +640,28 @@ tnmc_status tnmc_launch_logq_grad(const tnmc_env* env, int64_t B, const int8_t* 
   const size_t gsz = (size_t)d.Lx * d.Ly * d.P * 2 * d.P;
   TNMC_CUDA_TRY(cudaMemsetAsync(grad, 0, gsz * sizeof(float), stream));
   if (B == 0) return TNMC_OK;
-  const int W = (d.Lx + 31) / 32;
-  int dev = 0, max_optin = 0;
+  int dev = 0, max_optin = 0, nsm = 0;
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  auto smem_of = [&](int nt) {
-    return (size_t)7 * d.P * (nt + 1) * sizeof(float) + (size_t)2 * W * nt * sizeof(uint32_t);
-  };
-  int nsm = 0;
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  // 128 samples per CTA; 64 when P > 52 (shared memory) or when 128 would leave SMs idle
-  const int kNT = (smem_of(128) <= (size_t)max_optin && (B + 127) / 128 >= 2 * (int64_t)nsm) ? 128 : 64;
-  const size_t smem = smem_of(kNT);
+  const size_t smem = grad_smem(d.P, d.Lx).total;
   if (smem > (size_t)max_optin) {
     tnmc_set_error("gradient kernel needs %zu bytes of shared memory (device allows %d)", smem, max_optin);
     return TNMC_E_UNSUPPORTED;
   }
-  if (kNT == 128)
-    TNMC_CUDA_TRY(cudaFuncSetAttribute(logq_grad_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  else
-    TNMC_CUDA_TRY(cudaFuncSetAttribute(logq_grad_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int64_t ntiles = (B + kNT - 1) / kNT;
-  const size_t per_cta = (size_t)3 * (d.Lx + 1) * d.P * kNT + (size_t)4 * d.Lx * kNT;
-  const size_t need = (size_t)ntiles * per_cta * sizeof(float);
+  TNMC_CUDA_TRY(cudaFuncSetAttribute(logq_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int per_sm = 0;
+  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, logq_grad_kernel, kGThreads, smem));
+  int64_t grid = (B + kGT - 1) / kGT;
+  if (grid > (int64_t)nsm * (per_sm < 1 ? 1 : per_sm)) grid = (int64_t)nsm * (per_sm < 1 ? 1 : per_sm);
   tnmc_env* me = const_cast<tnmc_env*>(env);
   {
-    const tnmc_status gs = grow_scratch(me, need, stream, "gradient");
+    const tnmc_status gs = grow_scratch(me, (size_t)grid * grad_cta_floats(d.P, d.Lx) * sizeof(float), stream, "gradient");
     if (gs != TNMC_OK) return gs;
   }
   GradArgs a;
   a.e = d;
-  a.L = d.L32;
+  a.K = d.K32;
   a.Rt = d.R32;
   a.fe = d.fe32;
   a.B = B;
@@ -289,8 +669,7 @@ tnmc_status tnmc_launch_logq_grad(const tnmc_env* env, int64_t B, const int8_t* 
   a.weights = weights;
   a.grad = grad;
   a.scratch = static_cast<float*>(me->scratch.ptr);
-  if (kNT == 128) logq_grad_kernel<128><<<(unsigned)ntiles, 128, smem, stream>>>(a);
-  else logq_grad_kernel<64><<<(unsigned)ntiles, 64, smem, stream>>>(a);
+  logq_grad_kernel<<<(unsigned)grid, kGThreads, smem, stream>>>(a);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }
