@@ -280,6 +280,177 @@ __global__ void __launch_bounds__(32 * kScanWarps)
   }
 }
 
+// The scan with one CTA per chain, for few chains and many proposals, where one warp would
+// expose the dependent latency of every proposal.  An accepted proposal's successor does not
+// depend on how it was reached, so the accepted proposals of a block of up to kCtaBlock form a
+// linked list that is built in parallel:
+//   1. next[j]: the first m > j that a chain at proposal j accepts, by the bands, for every j at
+//      once (unknown where it is not within kCtaLook proposals or a band leaves it open);
+//   2. per chunk of 32 proposals, backwards: exit[j], the first list element beyond the chunk
+//      (or the element of the chunk whose successor is unknown);
+//   3. one warp walks the list chunk by chunk through exit[], and resolves an unknown successor
+//      by testing 32 proposals at a time, with the FP64 rule where the band leaves it open;
+//   4. every chunk marks its part of the list from the element the walk entered it by.
+// Decisions are those of the sequential rule.  One chain of 10^4 proposals: 345 us with one
+// warp, 27 us with one CTA (the walk, about 45 cycles per chunk, is half of it).
+constexpr int kCtaBlock = 4096;
+constexpr int kCtaChunk = 32;
+constexpr int kCtaLook = 8;
+constexpr int kCtaThreads = 128;
+// A CTA takes a few thousand cycles whatever T is, a warp about 83 per proposal: worth it from
+// T = 256 on (2048 chains of 128: 46.7 us against 46.0), while the CTAs of all chains fit the SMs in a few waves.
+constexpr int64_t kCtaMinT = 256, kCtaMaxChains = 2048;
+
+inline __host__ __device__ size_t mh_cta_smem(int nb) {
+  return (size_t)nb * (3 * sizeof(int64_t) + 2 * sizeof(int) + 1) + (size_t)(nb / kCtaChunk) * (2 * sizeof(int));
+}
+
+// index of proposal j in the link arrays: chunks start one bank apart
+__device__ __forceinline__ int mh_at(int j) { return j + (j >> 5); }
+
+__global__ void __launch_bounds__(kCtaThreads)
+    mh_scan_cta_kernel(int64_t T, int nb, double beta, uint64_t seed, uint64_t step_offset,
+                       const double* __restrict__ prop_logq, const double* __restrict__ prop_E,
+                       const int64_t* __restrict__ band_lo, const int64_t* __restrict__ band_hi,
+                       const int64_t* __restrict__ key_w, double* __restrict__ chain_logq,
+                       double* __restrict__ chain_E, uint8_t* __restrict__ accepted, int64_t* __restrict__ last,
+                       int64_t* n_accepted) {
+  extern __shared__ __align__(16) unsigned char sm_scan[];
+  __shared__ int s_last, s_count;
+  __shared__ ScanState s_state;
+  const int nchunk = nb / kCtaChunk;
+  int64_t* lo = reinterpret_cast<int64_t*>(sm_scan);
+  int64_t* hi = lo + nb;
+  int64_t* w = hi + nb;
+  int* nxt = reinterpret_cast<int*>(w + nb);       // [nb + nchunk]
+  int* ext = nxt + nb + nchunk;                    // [nb + nchunk]
+  uint8_t* flag = reinterpret_cast<uint8_t*>(ext + nb + nchunk);   // [nb]
+  __shared__ int entry[kCtaBlock / kCtaChunk];
+  const int64_t chain = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) s_state = mh_scan_start(beta, chain_logq[chain], chain_E[chain]);
+  int64_t lastt = -1, total = 0;       // thread 0
+  for (int64_t base = 0; base < T; base += nb) {
+    const int n = (T - base) < nb ? (int)(T - base) : nb;
+    const int64_t row = chain * T + base;
+    __syncthreads();
+    for (int j = tid; j < n; j += kCtaThreads) {
+      lo[j] = band_lo[row + j];
+      hi[j] = band_hi[row + j];
+      w[j] = key_w[row + j];
+      flag[j] = 0;
+    }
+    if (tid < nchunk) entry[tid] = -1;
+    if (tid == 0) {
+      s_last = -1;
+      s_count = 0;
+    }
+    __syncthreads();
+    for (int j = tid; j < n; j += kCtaThreads) {
+      const int64_t k = w[j];
+      int r = -1;
+      for (int m = j + 1; m <= j + kCtaLook; ++m) {
+        if (m >= n) {
+          r = n;
+          break;
+        }
+        if (k <= lo[m]) {
+          r = m;
+          break;
+        }
+        if (k < hi[m]) break;
+      }
+      nxt[mh_at(j)] = r;
+    }
+    __syncthreads();
+    for (int q = tid; q * kCtaChunk < n; q += kCtaThreads) {
+      const int j0 = q * kCtaChunk, j1 = min(j0 + kCtaChunk, n);
+      for (int j = j1 - 1; j >= j0; --j) {
+        const int e = nxt[mh_at(j)];
+        ext[mh_at(j)] = e < 0 ? -1 - j : e >= j1 ? e : ext[mh_at(e)];
+      }
+    }
+    __syncthreads();
+    if (tid < 32) {
+      // the first proposal m >= m0 that a chain in state st accepts (n: none)
+      auto search = [&](const ScanState& st, int m0) -> int {
+        while (m0 < n) {
+          const int m = m0 + lane;
+          bool a = false, open = false;
+          if (m < n) {
+            if (st.slow) {
+              a = mh_exact(beta, seed, step_offset + (uint64_t)(base + m), (uint32_t)chain, prop_logq[row + m],
+                           prop_E[row + m], mh_unkey(st.kc), st.start);
+            } else {
+              a = st.kc <= lo[m];
+              open = !a && st.kc < hi[m];
+            }
+          }
+          const unsigned any = __ballot_sync(0xffffffffu, a || open);
+          if (any == 0) {
+            m0 += 32;
+            continue;
+          }
+          const int f = __ffs(any) - 1;
+          if (lane == f && open)
+            a = mh_exact(beta, seed, step_offset + (uint64_t)(base + m), (uint32_t)chain, prop_logq[row + m],
+                         prop_E[row + m], mh_unkey(st.kc), false);
+          if (__shfl_sync(0xffffffffu, (int)a, f)) return m0 + f;
+          m0 += f + 1;
+        }
+        return n;
+      };
+      int e = search(s_state, 0);
+      if (e < n && lane == 0) entry[e / kCtaChunk] = e;
+      while (e < n) {
+        int x = ext[mh_at(e)];
+        if (x < 0) {
+          const int j = -1 - x;       // the element whose successor is unknown
+          const ScanState st{w[j], false, false};
+          x = search(st, j + 1);
+          if (lane == 0) nxt[mh_at(j)] = x;
+          if (x < n && x / kCtaChunk == j / kCtaChunk) {      // the list goes on within the chunk
+            e = x;
+            continue;
+          }
+        }
+        e = x;
+        if (e < n && lane == 0) entry[e / kCtaChunk] = e;
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q * kCtaChunk < n; q += kCtaThreads) {
+      const int j1 = min((q + 1) * kCtaChunk, n);
+      int cnt = 0, lj = -1;
+      for (int j = entry[q]; j >= 0 && j < j1; j = nxt[mh_at(j)]) {
+        flag[j] = 1;
+        lj = j;
+        ++cnt;
+      }
+      if (cnt) {
+        atomicAdd(&s_count, cnt);
+        atomicMax(&s_last, lj);
+      }
+    }
+    __syncthreads();
+    if (accepted)
+      for (int j = tid; j < n; j += kCtaThreads) accepted[row + j] = flag[j];
+    if (tid == 0 && s_last >= 0) {
+      lastt = row + s_last;
+      total += s_count;
+      s_state = ScanState{w[s_last], false, false};
+    }
+  }
+  if (tid == 0) {
+    if (lastt >= 0) {
+      chain_logq[chain] = prop_logq[lastt];
+      chain_E[chain] = prop_E[lastt];
+    }
+    last[chain] = lastt;
+    if (n_accepted && total) atomicAdd(reinterpret_cast<unsigned long long*>(n_accepted), (unsigned long long)total);
+  }
+}
+
 // Copy the last accepted proposal of each chain into the chain state (one CTA per chain).
 __global__ void mh_copy_kernel(int64_t C, int64_t n, const int64_t* last, const int8_t* __restrict__ prop,
                                int8_t* chain) {
@@ -336,7 +507,14 @@ tnmc_status tnmc_launch_mh_core(int64_t n, double beta, const tnmc::Allocator& a
                                             key_w);
   TNMC_CUDA_TRY(cudaGetLastError());
   const int threads = 128;   // 4 warps: the warp form's shared-memory layout
-  if (C <= 65536) {   // one warp per chain
+  if (C <= kCtaMaxChains && T >= kCtaMinT) {   // one CTA per chain
+    const int nb = T < kCtaBlock ? (int)((T + kCtaChunk - 1) / kCtaChunk) * kCtaChunk : kCtaBlock;
+    const size_t smem = mh_cta_smem(nb);
+    TNMC_CUDA_TRY(cudaFuncSetAttribute(mh_scan_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    mh_scan_cta_kernel<<<(unsigned)C, kCtaThreads, smem, stream>>>(T, nb, beta, seed, step_offset, prop_logq,
+                                                                   prop_energy, band_lo, band_hi, key_w, chain_logq,
+                                                                   chain_energy, accepted, last, n_accepted);
+  } else if (C <= 65536) {   // one warp per chain
     const int64_t blocks = (C * 32 + threads - 1) / threads;
     mh_scan_warp_kernel<<<(unsigned)blocks, threads, 0, stream>>>(C, T, beta, seed, step_offset, prop_logq,
                                                                   prop_energy, band_lo, band_hi, key_w, chain_logq,
