@@ -150,7 +150,6 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
   const size_t oK32 = (mask & (1 << TNMC_F32)) ? take(tens * 4) : 0;
   const size_t oL16 = (mask & (1 << TNMC_BF16)) ? take(ntens * tnmc_tc_tile_bytes()) : 0;
   const size_t oR16 = (mask & (1 << TNMC_BF16)) ? take(ntens * tnmc_tc_tile_bytes()) : 0;
-  const size_t oh32 = take(nh * 4), oJh32 = take((nJh ? nJh : 1) * 4), oJv32 = take((nJv ? nJv : 1) * 4);
   const size_t ols = take((size_t)Ly * 8), osv = take((size_t)Ly * (Lx + 1) * P * 8);
   const size_t odisc = take((size_t)Ly * (Lx + 1) * 8), ologZ = take(8), ostat = take(8);
   const size_t total = off;
@@ -206,9 +205,6 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
   env->discarded = reinterpret_cast<double*>(base + odisc);
   env->logZ = reinterpret_cast<double*>(base + ologZ);
   env->esz = reinterpret_cast<int32_t*>(base + oesz);
-  env->h32 = reinterpret_cast<float*>(base + oh32);
-  env->Jh32 = reinterpret_cast<float*>(base + oJh32);
-  env->Jv32 = reinterpret_cast<float*>(base + oJv32);
 
   d.qJh = reinterpret_cast<const int64_t*>(base + oqJh);
   d.qJv = reinterpret_cast<const int64_t*>(base + oqJv);

@@ -85,9 +85,6 @@ struct tnmc_env {
   double* discarded = nullptr;   // [Ly][Lx+1]
   double* logZ = nullptr;        // scalar
   int32_t* esz = nullptr;        // [Ly][Lx+1] even-sector size per bond (Z2 builder)
-  float* h32 = nullptr;          // FP32 couplings for the tensor-core sampler's energy
-  float* Jh32 = nullptr;
-  float* Jv32 = nullptr;
   tnmc::Scratch scratch;         // sampler scratch (grown on demand)
   tnmc::Allocator alloc;         // the hook current when the env was created
 };
@@ -150,6 +147,17 @@ __device__ inline bool draw_plus(float pplus, uint64_t x) {
   if (pplus >= 1.0f) return true;
   if (!(pplus > 0.0f)) return false;
   return x < __float2ull_rz(pplus * 0x1.0p64f);
+}
+
+// +1 iff x < floor(p 2^64) (draw_plus), from the bits of p
+__device__ __forceinline__ bool draw_plus_bits(float p, uint64_t x) {
+  const int b = __float_as_int(p);
+  if (b >= 0x3f800000) return true;                  // p >= 1
+  if (b <= 0) return false;                            // p <= 0
+  const int sh = (b >> 23) - 86;                       // p 2^64 = mantissa 2^sh, sh <= 40
+  const uint64_t m = (uint64_t)((b & 0x7fffff) | ((b >> 23) ? 0x800000 : 0));
+  const uint64_t t = sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ull);
+  return x < t;
 }
 
 inline int pad4(int x) { return (x + 3) & ~3; }

@@ -66,17 +66,6 @@ __device__ __forceinline__ int exponent_f32(int bits) {
   return (ex == 0 || ex == 255) ? 0 : min(ex - 127, 126);
 }
 
-// +1 iff x < floor(p 2^64) (draw_plus), from the bits of p
-__device__ __forceinline__ bool draw_plus_bits(float p, uint64_t x) {
-  const int b = __float_as_int(p);
-  if (b >= 0x3f800000) return true;                  // p >= 1
-  if (b <= 0) return false;                            // p <= 0
-  const int sh = (b >> 23) - 86;                       // p 2^64 = mantissa 2^sh, sh <= 40
-  const uint64_t m = (uint64_t)((b & 0x7fffff) | ((b >> 23) ? 0x800000 : 0));
-  const uint64_t t = sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ull);
-  return x < t;
-}
-
 // N consecutive floats from an address aligned to gcd(N, 4) floats
 template <int N>
 __device__ __forceinline__ void load_run(const float* p, float* o) {
