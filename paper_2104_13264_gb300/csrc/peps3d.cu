@@ -21,7 +21,8 @@
 // left vector Lambda (sites < x drawn), clamped at zero and normalised, drawn with the
 // Philox word of site (z Ly + y) Lx + x.  The per-sample scratch lives in HBM with the
 // sample index fastest (element i of sample b at base[i * Bc + b]), so every load and
-// store of a warp is coalesced.
+// store of a warp is coalesced; small batches keep a sample's working matrices in shared
+// memory instead (sample3d_kernel<T, true>).
 #include <math.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -68,6 +69,15 @@ struct V {
   __device__ __forceinline__ V at(int64_t off) const { return V{p + off * s, s}; }
 };
 
+// The same view over a warp's shared memory: element i of lane l at p[32 i] (p includes l), so
+// every access of a warp is conflict free.
+template <typename T>
+struct VS {
+  T* p;
+  __device__ __forceinline__ T& operator[](int64_t i) const { return p[32 * (int)i]; }
+  __device__ __forceinline__ VS at(int64_t off) const { return VS{p + 32 * (int)off}; }
+};
+
 template <typename T>
 struct Tol3;
 template <>
@@ -83,8 +93,8 @@ struct Tol3<float> {
 // On return J's rows are orthogonal and d[i] holds their 2-norms.  Rows below `null`
 // of the largest are left out of the rotations.  Returns false when the last sweep
 // still rotated.
-template <typename T>
-__device__ bool orth_rows(V<T> J, int m, int n, V<T> d) {
+template <typename T, typename VJ>
+__device__ bool orth_rows(VJ J, int m, int n, VJ d) {
   bool converged = false;
   for (int sweep = 0; sweep < kSweeps3 && !converged; ++sweep) {
     T dmax = 0;
@@ -128,8 +138,8 @@ __device__ bool orth_rows(V<T> J, int m, int n, V<T> d) {
 }
 
 // sel[0..k) = the k rows of largest norm (descending; ties by index).
-template <typename T>
-__device__ void select_rows(V<T> d, int m, int k, int* sel) {
+template <typename T, typename VJ>
+__device__ void select_rows(VJ d, int m, int k, int* sel) {
   for (int i = 0; i < m; ++i) {
     int rank = 0;
     const T di = d[i];
@@ -215,10 +225,10 @@ __device__ int mps_compress(V<T> M, int64_t cap, int ns, int* dl, const int* pp,
     V<T> Mi = M.at(i * cap);
     if (a > kMaxRows3) return TNMC_E_NUMERIC;
     for (int e = 0; e < a * len; ++e) J[e] = Mi[e];
-    if (!orth_rows(J, a, len, d)) err = TNMC_E_NUMERIC;
+    if (!orth_rows<T>(J, a, len, d)) err = TNMC_E_NUMERIC;
     int k = a < len ? a : len;
     k = kmax < k ? kmax : k;
-    select_rows(d, a, k, sel);
+    select_rows<T>(d, a, k, sel);
     const T smax = d[sel[0]];
     if (!(smax > 0) || !isfinite((double)smax)) return TNMC_E_NUMERIC;
     for (int j = 0; j < k; ++j) {
@@ -255,6 +265,128 @@ __device__ int mps_compress(V<T> M, int64_t cap, int ns, int* dl, const int* pp,
     if (!(nrm > 0) || !isfinite((double)nrm)) return TNMC_E_NUMERIC;
     const T inv = T(1) / nrm;
     for (int e = 0; e < n0; ++e) M[e] *= inv;
+    lg += log((double)nrm);
+  }
+  *logs = lg;
+  return err;
+}
+
+// mps_compress with its matrices in shared memory: the same operations in the same order, but
+// the site being worked on stays in C (the sites in M are read once and written once per sweep).
+template <typename T>
+__device__ int mps_compress_shared(V<T> M, int64_t cap, int ns, int* dl, const int* pp, int* dr, int kmax, VS<T> J,
+                                   VS<T> d, VS<T> sm, VS<T> tmp, VS<T> C, double* logs) {
+  int sel[kMaxRows3];
+  int err = 0;
+  double lg = 0.0;
+  {
+    const int n0 = dl[0] * pp[0] * dr[0];
+    for (int e = 0; e < n0; ++e) C[e] = M[e];
+  }
+  for (int i = 0; i + 1 < ns; ++i) {
+    const int a = dl[i], p = pp[i], b = dr[i], len = a * p;
+    V<T> Mi = M.at(i * cap);
+    const int k = len < b ? len : b;
+    for (int e = 0; e < k * b; ++e) sm[e] = T(0);
+    int acc = 0;
+    for (int j = 0; j < b; ++j) {
+      T nx = 0;
+      for (int x = 0; x < len; ++x) {
+        const T v = C[x * b + j];
+        tmp[x] = v;
+        nx += v * v;
+      }
+      for (int pass = 0; pass < 2; ++pass)
+        for (int q = 0; q < acc; ++q) {
+          T r = 0;
+          for (int x = 0; x < len; ++x) r += J[q * len + x] * tmp[x];
+          for (int x = 0; x < len; ++x) tmp[x] -= r * J[q * len + x];
+          sm[q * b + j] += r;
+        }
+      T nv = 0;
+      for (int x = 0; x < len; ++x) nv += tmp[x] * tmp[x];
+      nv = sqrt(nv);
+      if (acc < k && nv > Tol3<T>::qr * sqrt(nx) && nv > 0) {
+        const T inv = T(1) / nv;
+        for (int x = 0; x < len; ++x) J[acc * len + x] = tmp[x] * inv;
+        sm[acc * b + j] = nv;
+        ++acc;
+      }
+    }
+    for (int q = acc; q < k; ++q)
+      for (int x = 0; x < len; ++x) J[q * len + x] = T(0);
+    T sc = 0;
+    for (int e = 0; e < k * b; ++e) {
+      const T aa = sm[e] < 0 ? -sm[e] : sm[e];
+      sc = aa > sc ? aa : sc;
+    }
+    if (!(sc > 0) || !isfinite((double)sc)) return TNMC_E_NUMERIC;
+    lg += log((double)sc);
+    for (int q = 0; q < k; ++q)
+      for (int x = 0; x < len; ++x) Mi[(int64_t)x * k + q] = J[q * len + x];
+    V<T> Mn = M.at((i + 1) * cap);
+    const int rest = pp[i + 1] * dr[i + 1];
+    const T isc = T(1) / sc;
+    for (int e = 0; e < b * rest; ++e) C[e] = Mn[e];
+    for (int j = 0; j < k; ++j)
+      for (int y = 0; y < rest; ++y) {
+        T acc = 0;
+        for (int c = 0; c < b; ++c) acc += sm[j * b + c] * C[c * rest + y];
+        tmp[j * rest + y] = acc * isc;
+      }
+    for (int e = 0; e < k * rest; ++e) C[e] = tmp[e];
+    dr[i] = k;
+    dl[i + 1] = k;
+  }
+  for (int i = ns - 1; i >= 1; --i) {
+    const int a = dl[i], p = pp[i], b = dr[i], len = p * b;
+    V<T> Mi = M.at(i * cap);
+    if (a > kMaxRows3) return TNMC_E_NUMERIC;
+    for (int e = 0; e < a * len; ++e) J[e] = C[e];
+    if (!orth_rows<T>(J, a, len, d)) err = TNMC_E_NUMERIC;
+    int k = a < len ? a : len;
+    k = kmax < k ? kmax : k;
+    select_rows<T>(d, a, k, sel);
+    const T smax = d[sel[0]];
+    if (!(smax > 0) || !isfinite((double)smax)) return TNMC_E_NUMERIC;
+    for (int j = 0; j < k; ++j) {
+      const T nj = d[sel[j]];
+      const T inv = nj > Tol3<T>::null * smax ? T(1) / nj : T(0);
+      for (int y = 0; y < len; ++y) {
+        const T v = J[sel[j] * len + y] * inv;
+        tmp[j * len + y] = v;
+        Mi[(int64_t)j * len + y] = v;
+      }
+    }
+    const T is = T(1) / smax;
+    for (int r = 0; r < a; ++r)
+      for (int j = 0; j < k; ++j) {
+        T acc = 0;
+        for (int y = 0; y < len; ++y) acc += C[r * len + y] * tmp[j * len + y];
+        sm[r * k + j] = acc * is;
+      }
+    lg += log((double)smax);
+    V<T> Mp = M.at((i - 1) * cap);
+    const int rows = dl[i - 1] * pp[i - 1];
+    for (int e = 0; e < rows * a; ++e) C[e] = Mp[e];
+    for (int z = 0; z < rows; ++z)
+      for (int j = 0; j < k; ++j) {
+        T acc = 0;
+        for (int r = 0; r < a; ++r) acc += C[z * a + r] * sm[r * k + j];
+        tmp[z * k + j] = acc;
+      }
+    for (int e = 0; e < rows * k; ++e) C[e] = tmp[e];
+    dl[i] = k;
+    dr[i - 1] = k;
+  }
+  {
+    const int n0 = dl[0] * pp[0] * dr[0];
+    T s = 0;
+    for (int e = 0; e < n0; ++e) s += C[e] * C[e];
+    const T nrm = sqrt(s);
+    if (!(nrm > 0) || !isfinite((double)nrm)) return TNMC_E_NUMERIC;
+    const T inv = T(1) / nrm;
+    for (int e = 0; e < n0; ++e) M[e] = C[e] * inv;
     lg += log((double)nrm);
   }
   *logs = lg;
@@ -584,17 +716,41 @@ __device__ __forceinline__ T absT(T v) {
   return v < 0 ? -v : v;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128, 4) sample3d_kernel(Samp3 a) {
+// Elements of one sample's shared-memory slice (SH form): J and sm, which U1 and U2 overlay, d,
+// tmp, and the site being compressed, which lam overlays.
+__host__ __device__ inline int64_t shared3_elems(int D, int chi) {
+  const int64_t K = (int64_t)D * chi;
+  return K * K * D + K * K + K + 2 * K * D * K;
+}
+
+// SH: one warp per CTA with the working matrices in shared memory (32 slices); otherwise
+// 128 threads per CTA with everything in the global scratch.  One thread's sample is a chain of
+// small products and Jacobi sweeps: from global scratch every operand is an L1 or L2 access
+// (921 words a sample at D chi = 8 overflow L1), from shared memory a conflict-free load.
+template <typename T, bool SH>
+__global__ void __launch_bounds__(SH ? 32 : 128, SH ? 2 : 4) sample3d_kernel(Samp3 a) {
   const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (b >= a.Bc) return;
   const int64_t g = a.b0 + b;
   const int Lx = a.Lx, Ly = a.Ly, Lz = a.Lz, D = a.D, chi = a.chi;
   const Lay3 o = lay3(Lx, Ly, D, chi);
   const V<T> base{static_cast<T*>(a.scr) + b, a.Bc};
-  const V<T> Bot = base.at(o.bot), Top = base.at(o.top), W = base.at(o.w), J = base.at(o.J), dv = base.at(o.d);
-  const V<T> sm = base.at(o.sm), tmp = base.at(o.tmp), R = base.at(o.R), lam = base.at(o.lam);
-  const V<T> U1 = base.at(o.U1), U2 = base.at(o.U2);
+  const V<T> Bot = base.at(o.bot), Top = base.at(o.top), W = base.at(o.w), R = base.at(o.R);
+  extern __shared__ __align__(16) unsigned char sm3_raw[];
+  const int64_t K3 = (int64_t)D * chi;
+  const VS<T> sh{reinterpret_cast<T*>(sm3_raw) + (threadIdx.x & 31)};
+  // working matrices: views of the warp's shared memory, or of the global scratch
+  auto view = [&](int64_t global_off, int64_t shared_off) {
+    if constexpr (SH) return sh.at(shared_off);
+    else return base.at(global_off);
+  };
+  const int64_t sJ = 0, sS = K3 * K3 * D, sD = sS + K3 * K3, sT = sD + K3, sC = sT + K3 * D * K3;
+  const auto J = view(o.J, sJ), sm = view(o.sm, sS), dv = view(o.d, sD), tmp = view(o.tmp, sT), lam = view(o.lam, sC);
+  const auto U1 = view(o.U1, 0), U2 = view(o.U2, K3 * K3);
+  auto compress = [&](int* wl, const int* wp, int* wr, double* lg) -> int {
+    if constexpr (SH) return mps_compress_shared<T>(W, o.capW, Lx, wl, wp, wr, chi, J, dv, sm, tmp, sh.at(sC), lg);
+    else return mps_compress<T>(W, o.capW, Lx, wl, wp, wr, chi, J, dv, sm, tmp, lg);
+  };
   const V<int32_t> botb{a.iscr + b, a.Bc};
   const T* A = static_cast<const T*>(a.A);
   const int64_t site_sz = 2LL * D * D * D * D;
@@ -635,7 +791,7 @@ __global__ void __launch_bounds__(128, 4) sample3d_kernel(Samp3 a) {
         wr[x] = ncol;
       }
       double lg;
-      const int e = mps_compress(W, o.capW, Lx, wl, wp, wr, chi, J, dv, sm, tmp, &lg);
+      const int e = compress(wl, wp, wr, &lg);
       err = err ? err : e;
       for (int x = 0; x < Lx; ++x) {
         const V<T> Bd = Bot.at(((int64_t)y * Lx + x) * o.capS);
@@ -805,7 +961,7 @@ __global__ void __launch_bounds__(128, 4) sample3d_kernel(Samp3 a) {
           wr[x] = ncol;
         }
         double lg;
-        const int e = mps_compress(W, o.capW, Lx, wl, wp, wr, chi, J, dv, sm, tmp, &lg);
+        const int e = compress(wl, wp, wr, &lg);
         err = err ? err : e;
         for (int x = 0; x < Lx; ++x) {
           const V<T> Tx = Top.at(x * o.capS), Wx = W.at(x * o.capW);
@@ -1611,7 +1767,7 @@ static tnmc_status run3d(const tnmc3d_env* env, int precision, int64_t B, uint64
   // thread per sample below.  Measured on the 16^3 bond-basis (2, 2) line (D chi = 8):
   // one thread 15.9 s per step, groups of 8 lanes 29.3 s, of 16 lanes 41.5 s (the per-step
   // reductions and syncs cost more than the lanes gain on 8-wide vectors); at D chi = 16 the
-  // warp form is the faster one.  TNMC_3D_KERNEL=thread|warp|group8|group16 overrides.
+  // warp form is the faster one.  TNMC_3D_KERNEL=thread|shared|warp|group8|group16 overrides (thread: global scratch).
   const WLay wl = wlay(env->Ds, env->chi);
   const size_t wbytes = wslice_bytes(wl, esz);
   int dev = 0, max_optin = 0;
@@ -1620,7 +1776,7 @@ static tnmc_status run3d(const tnmc3d_env* env, int precision, int64_t B, uint64
   const int64_t K = (int64_t)env->Ds * env->chi;
   int G = K >= 16 ? 32 : 0;
   const char* force = getenv("TNMC_3D_KERNEL");
-  if (force && force[0] == 't') G = 0;
+  if (force && (force[0] == 't' || force[0] == 's')) G = 0;
   if (force && force[0] == 'w') G = 32;
   if (force && strcmp(force, "group8") == 0) G = 8;
   if (force && strcmp(force, "group16") == 0) G = 16;
@@ -1633,7 +1789,28 @@ static tnmc_status run3d(const tnmc3d_env* env, int precision, int64_t B, uint64
     spb -= spb % per_warp;
     if (spb < per_warp) G = 0;
   }
-  tnmc_status st = TNMC_OK;
+  // one thread per sample: the working matrices in shared memory while one wave of one-warp CTAs
+  // holds the batch, or where at least 8 such CTAs fit an SM; else in the global scratch, whose
+  // 16 warps per SM then win.  Measured (global / shared, ms, FP32): 6^3 bond (2, 2), D chi = 8, two
+  // warps per SM: 8192 samples 93.5 / 61.7, 32768 131 / 245; spin (2, 2), D chi = 4: 8192 15.8 / 12.0,
+  // 65536 147 / 37; 5^3 spin (3, 4), D chi = 12, one warp: 1024 59.6 / 37.8, 8192 63.8 / 75.5.
+  size_t shbytes = 0;
+  auto shared_form = [&]() -> tnmc_status {
+    const size_t need = (size_t)shared3_elems(env->Ds, env->chi) * 32 * esz;
+    if (need > (size_t)max_optin) return TNMC_OK;
+    int per_sm = 0, nsm = 0;
+    TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    if (precision == TNMC_F64) {
+      TNMC_CUDA_TRY(cudaFuncSetAttribute(sample3d_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
+      TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample3d_kernel<double, true>, 32, need));
+    } else {
+      TNMC_CUDA_TRY(cudaFuncSetAttribute(sample3d_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
+      TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample3d_kernel<float, true>, 32, need));
+    }
+    if (per_sm >= 8 || (per_sm > 0 && (B <= (int64_t)nsm * per_sm * 32 || (force && force[0] == 's')))) shbytes = need;
+    return TNMC_OK;
+  };
+  tnmc_status st = (!G && !(force && force[0] == 't')) ? shared_form() : TNMC_OK;
   for (int64_t b0 = 0; b0 < B && st == TNMC_OK; b0 += Bc) {
     a.b0 = b0;
     a.Bc = (B - b0) < Bc ? (B - b0) : Bc;
@@ -1643,10 +1820,15 @@ static tnmc_status run3d(const tnmc3d_env* env, int precision, int64_t B, uint64
          : G == 16 ? (f64 ? launch_group<double, 16>(a, spb, wbytes, s) : launch_group<float, 16>(a, spb, wbytes, s))
                    : (f64 ? launch_group<double, 8>(a, spb, wbytes, s) : launch_group<float, 8>(a, spb, wbytes, s));
     } else {
-      const int threads = 128;
+      const int threads = shbytes ? 32 : 128;
       const unsigned blocks = (unsigned)((a.Bc + threads - 1) / threads);
-      if (precision == TNMC_F64) sample3d_kernel<double><<<blocks, threads, 0, s>>>(a);
-      else sample3d_kernel<float><<<blocks, threads, 0, s>>>(a);
+      if (precision == TNMC_F64) {
+        if (shbytes) sample3d_kernel<double, true><<<blocks, threads, shbytes, s>>>(a);
+        else sample3d_kernel<double, false><<<blocks, threads, 0, s>>>(a);
+      } else {
+        if (shbytes) sample3d_kernel<float, true><<<blocks, threads, shbytes, s>>>(a);
+        else sample3d_kernel<float, false><<<blocks, threads, 0, s>>>(a);
+      }
       if (cudaGetLastError() != cudaSuccess) {
         tnmc_set_error("3D sampler launch failed");
         st = TNMC_E_CUDA;
