@@ -58,12 +58,13 @@ inline __host__ __device__ size_t grad_cta_floats(int P, int Lx) {
 }
 
 // Shared memory: the tensor ring, two buffer sets of 6 P vector rows, partial maxima and
-// weights, field factors, bond dimensions and spin masks of the row, sample flags.
+// weights, spin masks of the row, sample flags, and if `staged` the row's field factors and
+// bond dimensions.
 struct GradSmem {
   int nbuf;
   size_t set, mpart, wpart, fer, bond, mask, ok, total;
 };
-inline __host__ __device__ GradSmem grad_smem(int P, int Lx) {
+inline __host__ __device__ GradSmem grad_smem(int P, int Lx, bool staged) {
   GradSmem m;
   m.nbuf = P > 32 ? 2 : 3;
   size_t o = ((size_t)m.nbuf * P * 2 * P + 128) * sizeof(float);
@@ -73,14 +74,14 @@ inline __host__ __device__ GradSmem grad_smem(int P, int Lx) {
   o += (size_t)2 * 4 * kGT * sizeof(float);
   m.wpart = o;
   o += (size_t)2 * 4 * 2 * kGT * sizeof(float);
-  m.fer = o;
-  o += (size_t)2 * Lx * sizeof(float);
-  m.bond = o;
-  o += (size_t)(Lx + 1) * sizeof(int);
   m.mask = o;
   o += (size_t)2 * Lx * sizeof(uint32_t);
   m.ok = o;
   o += kGT * sizeof(int);
+  m.fer = o;
+  if (staged) o += (size_t)2 * Lx * sizeof(float);
+  m.bond = o;
+  if (staged) o += (size_t)(Lx + 1) * sizeof(int);
   m.total = o;
   return m;
 }
@@ -218,20 +219,21 @@ __device__ __forceinline__ void site_gradient(const float* V, const float* W, co
   }
 }
 
+// STAGED: the row's field factors and bond dimensions in shared memory; rows too wide for that
+// (P = 64: more than 2630 columns) read them from global memory.
+template <bool STAGED>
 __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const unsigned kFull = 0xffffffffu;
   const int Lx = a.e.Lx, Ly = a.e.Ly, P = a.e.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sl = lane & 7, ol = (lane >> 3) + 4 * warp;      // samples 4 sl .. 4 sl + 3, outputs XB ol ..
-  const GradSmem lay = grad_smem(P, Lx);
+  const GradSmem lay = grad_smem(P, Lx, STAGED);
   float* ring = reinterpret_cast<float*>(smem_raw);
   float* set0 = reinterpret_cast<float*>(smem_raw + lay.set);
   const size_t set_sz = (size_t)6 * P * kGStride;
   float* mpart = reinterpret_cast<float*>(smem_raw + lay.mpart);     // [2][4][kGT]
   float* wpart = reinterpret_cast<float*>(smem_raw + lay.wpart);     // [2][4][2][kGT]
-  float* fer = reinterpret_cast<float*>(smem_raw + lay.fer);
-  int* bond = reinterpret_cast<int*>(smem_raw + lay.bond);
   uint32_t* prev = reinterpret_cast<uint32_t*>(smem_raw + lay.mask);
   uint32_t* cur = prev + Lx;
   int* okf = reinterpret_cast<int*>(smem_raw + lay.ok);
@@ -306,8 +308,16 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
 
     for (int r = 0; r < Ly; ++r) {
       __syncthreads();
-      for (int c = tid; c <= Lx; c += kGThreads) bond[c] = a.e.bond[r * (Lx + 1) + c];
-      for (int c = tid; c < 2 * Lx; c += kGThreads) fer[c] = r == 0 ? 1.0f : a.fe[(size_t)r * Lx * 2 + c];
+      const int* bond = a.e.bond + (size_t)r * (Lx + 1);
+      const float* fer = a.fe + (size_t)r * Lx * 2;       // 1 on row 0
+      if constexpr (STAGED) {
+        int* sbond = reinterpret_cast<int*>(smem_raw + lay.bond);
+        float* sfer = reinterpret_cast<float*>(smem_raw + lay.fer);
+        for (int c = tid; c <= Lx; c += kGThreads) sbond[c] = bond[c];
+        for (int c = tid; c < 2 * Lx; c += kGThreads) sfer[c] = fer[c];
+        bond = sbond;
+        fer = sfer;
+      }
       for (int c = tid; c < Lx; c += kGThreads) {
         const int8_t* src = a.spins + (size_t)base * n + (size_t)r * Lx + c;
         uint32_t m = 0;
@@ -644,14 +654,16 @@ tnmc_status tnmc_launch_logq_grad(const tnmc_env* env, int64_t B, const int8_t* 
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const size_t smem = grad_smem(d.P, d.Lx).total;
+  const bool staged = grad_smem(d.P, d.Lx, true).total <= (size_t)max_optin;
+  const size_t smem = grad_smem(d.P, d.Lx, staged).total;
   if (smem > (size_t)max_optin) {
     tnmc_set_error("gradient kernel needs %zu bytes of shared memory (device allows %d)", smem, max_optin);
     return TNMC_E_UNSUPPORTED;
   }
-  TNMC_CUDA_TRY(cudaFuncSetAttribute(logq_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  auto kern = staged ? logq_grad_kernel<true> : logq_grad_kernel<false>;
+  TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, logq_grad_kernel, kGThreads, smem));
+  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGThreads, smem));
   int64_t grid = (B + kGT - 1) / kGT;
   if (grid > (int64_t)nsm * (per_sm < 1 ? 1 : per_sm)) grid = (int64_t)nsm * (per_sm < 1 ? 1 : per_sm);
   tnmc_env* me = const_cast<tnmc_env*>(env);
@@ -669,7 +681,7 @@ tnmc_status tnmc_launch_logq_grad(const tnmc_env* env, int64_t B, const int8_t* 
   a.weights = weights;
   a.grad = grad;
   a.scratch = static_cast<float*>(me->scratch.ptr);
-  logq_grad_kernel<<<(unsigned)grid, kGThreads, smem, stream>>>(a);
+  kern<<<(unsigned)grid, kGThreads, smem, stream>>>(a);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }

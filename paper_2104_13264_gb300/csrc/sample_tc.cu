@@ -53,6 +53,7 @@ constexpr int kK = 64;              // padded bond dimension (UMMA K per site)
 constexpr int kN = 128;             // 2 x 64 outputs (UMMA N)
 constexpr uint32_t kTileBytes = kN * kK * 2;   // 16 KiB: one BF16 operand tile
 constexpr uint32_t kStageBytes = 2 * kTileBytes;   // hi + lo tiles of one (r, c)
+constexpr int kMaxCols = 3968;      // widest row
 constexpr int kStages = 2;          // environment tiles in flight
 constexpr uint32_t kRBytes = kTile * kK * 4;   // 32 KiB: R_{c+1} of the tile, FP32
 constexpr uint32_t kTmemCols = 256; // 128 accumulator columns, 32 + 32 of the A operand (hi, lo)
@@ -117,6 +118,10 @@ __device__ inline void pair_sync(int warp) {
   asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory");
 }
 
+// STAGED: the row's field factors and the masks of its own spins in shared memory.  Otherwise
+// the factors are read from the environment and the masks kept behind the stacks in global
+// scratch.
+template <bool STAGED>
 __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -131,9 +136,10 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
   float* xmb = xw + 4 * kTile;                      // right steps: [2 halves][128] partial max
   const int Lx = a.e.Lx, Ly = a.e.Ly;
   uint32_t* xs = reinterpret_cast<uint32_t*>(xw + 8 * kTile);   // [2 pairs][2 sites][2][128]: 64-bit uniforms
-  float* fe_row = reinterpret_cast<float*>(xs + 8 * kTile);     // [Lx][2]: field factors of the row
-  uint32_t* prev = reinterpret_cast<uint32_t*>(fe_row + 2 * Lx);   // [Lx][4]: spins of the row above, one bit a sample
-  uint32_t* cur = prev + 4 * Lx;
+  uint32_t* prev = xs + 8 * kTile;                              // [Lx][4]: spins of the row above, one bit a sample
+  uint32_t* cur = STAGED ? prev + 4 * Lx
+                         : reinterpret_cast<uint32_t*>(a.stack + (size_t)gridDim.x * Lx * (2 * 8 * kTile)) +
+                               (size_t)blockIdx.x * 4 * Lx;
 
   const int tid = threadIdx.x, warp = tid >> 5;
   const bool ctrl = warp >= 8;                          // the UMMA warp (8) and the producer warp (9)
@@ -215,7 +221,12 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
       }
     };
     for (int r = 0; r < Ly && !abort; ++r) {
-      for (int q = tid; q < 2 * Lx; q += kThreads) fe_row[q] = r == 0 ? 1.0f : a.fe[(size_t)r * Lx * 2 + q];
+      const float* fe_row = a.fe + (size_t)r * Lx * 2;     // [Lx][2]: field factors of the row; 1 on row 0
+      if constexpr (STAGED) {
+        float* sfe = reinterpret_cast<float*>(cur + 4 * Lx);
+        for (int q = tid; q < 2 * Lx; q += kThreads) sfe[q] = fe_row[q];
+        fe_row = sfe;
+      }
       if (a.spins_in && warp < 4) {
         const int64_t b0 = tile * kTile + 32 * warp;
         const int ns = (a.B - b0) < 32 ? (int)(a.B - b0) : 32;
@@ -586,28 +597,40 @@ tnmc_status tnmc_launch_sample_tc(const tnmc_env* env, int64_t B, uint64_t seed,
     tnmc_set_error("the tensor-core sampler supports chi <= 64");
     return TNMC_E_UNSUPPORTED;
   }
-  const size_t smem = 1024 + kStages * kStageBytes + kRBytes + (kStages + 1) * 8 + 24 +
-                      (size_t)16 * kTile * sizeof(float) + (size_t)10 * d.Lx * sizeof(uint32_t);
-  int dev = 0, nsm = 0, max_optin = 0;
+  int dev = 0, nsm = 0, max_optin = 0, smem_sm = 0;
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
+  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  if (d.Lx > kMaxCols) {
+    tnmc_set_error("the tensor-core sampler supports rows of at most %d sites", kMaxCols);
+    return TNMC_E_UNSUPPORTED;
+  }
+  size_t smem = 1024 + kStages * kStageBytes + kRBytes + (kStages + 1) * 8 + 24 +
+                (size_t)16 * kTile * sizeof(float) + (size_t)4 * d.Lx * sizeof(uint32_t);
+  // Staged unless that does not fit (more than 3122 columns) or costs the SM its second CTA (204 to
+  // 509 columns).  Measured, chi 16, 6 rows, 65536 samples, staged / not: 96 columns 4.59 / 4.68 ms,
+  // 256 columns 18.2 (one CTA) / 12.5 (two), 600 columns 42.9 / 44.5.
+  const size_t row_bytes = (size_t)6 * d.Lx * sizeof(uint32_t);
+  const bool staged = smem + row_bytes <= (size_t)max_optin &&
+                      (2 * (smem + row_bytes + 1024) <= (size_t)smem_sm || 2 * (smem + 1024) > (size_t)smem_sm);
+  if (staged) smem += row_bytes;
   if (smem > (size_t)max_optin) {
     tnmc_set_error("tensor-core sampler needs %zu bytes of shared memory (device allows %d)", smem, max_optin);
     return TNMC_E_UNSUPPORTED;
   }
-  TNMC_CUDA_TRY(cudaFuncSetAttribute(sample_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  TNMC_CUDA_TRY(cudaFuncSetAttribute(sample_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+  auto kern = staged ? sample_tc_kernel<true> : sample_tc_kernel<false>;
+  TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared));
   int per_sm = 0;
-  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample_tc_kernel, kThreads, smem));
+  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
   {
     // cross-check the occupancy query against the shared-memory budget of an SM
-    int smem_sm = 0, regs_sm = 0;
-    TNMC_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    int regs_sm = 0;
     TNMC_CUDA_TRY(cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev));
     cudaFuncAttributes fa;
-    TNMC_CUDA_TRY(cudaFuncGetAttributes(&fa, sample_tc_kernel));
+    TNMC_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
     const int by_smem = smem_sm / (int)(smem + 1024);
     const int by_regs = regs_sm / (((fa.numRegs + 7) & ~7) * kThreads);
     const int est = by_smem < by_regs ? by_smem : by_regs;
@@ -618,7 +641,7 @@ tnmc_status tnmc_launch_sample_tc(const tnmc_env* env, int64_t B, uint64_t seed,
   const int64_t ntiles = (B + kTile - 1) / kTile;
   int64_t grid = (int64_t)nsm * per_sm;
   if (grid > ntiles) grid = ntiles;
-  const size_t need = (size_t)grid * d.Lx * kTile * kK * sizeof(float);
+  const size_t need = (size_t)grid * d.Lx * (kTile * kK * sizeof(float) + (staged ? 0 : 4 * sizeof(uint32_t)));
   tnmc_env* me = const_cast<tnmc_env*>(env);
   {
     const tnmc_status gs = grow_scratch(me, need, stream, "sampler");
@@ -645,7 +668,7 @@ tnmc_status tnmc_launch_sample_tc(const tnmc_env* env, int64_t B, uint64_t seed,
     const char* pl = getenv("TNMC_DEBUG_POLL_LIMIT");
     if (pl && *pl) a.poll_limit = (uint32_t)strtoul(pl, nullptr, 10);
   }
-  sample_tc_kernel<<<(unsigned)grid, kThreads, smem, stream>>>(a);
+  kern<<<(unsigned)grid, kThreads, smem, stream>>>(a);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }
