@@ -15,8 +15,8 @@
 //     sum from the masks, and log q a product with integer exponents (one log per sample), so
 //     that nothing per site runs on the FP64 pipe.
 // Measured against one thread per sample (128 per CTA): 32 x 32, chi = 16, 65536 samples 11.3 ->
-// 4.95 ms (25 % of the FFMA peak; 1.7 warps per scheduler issue 60 % of the cycles, a third of it
-// the ordered dot product, draws and stores); 24 x 45, chi = 32, 16384 samples 28.8 -> 4.5 ms.
+// 4.88 ms (25 % of the FFMA peak; 1.7 warps per scheduler: latency, a third of it the ordered dot
+// product, draws and stores); 24 x 45, chi = 32, 16384 samples 28.8 -> 4.4 ms.
 //
 // The products and sums that decide a draw are taken in the order of a plain loop over the
 // bonds (the dot product <U[s], R> is passed from output lane to output lane), so the results
@@ -27,6 +27,7 @@
 
 #include "common.cuh"
 #include "sample_args.cuh"
+#include "umma.cuh"
 
 namespace tnmc {
 namespace {
@@ -119,6 +120,10 @@ struct F32Lane {
 };
 
 // acc[s][j][b] = sum_k M[k][x0 + j][s] X[k][sample b], x0 = XB g, in the order k = 0, 1, ...
+// Paired FP32 FMAs halve the issue slots; the pairs run over the spins where the block has fewer
+// samples than tensor entries (one duplicated operand per sample instead of one per entry), else
+// over the samples.  Against single FMAs (chi 24 / 32): 65536 samples of 12 x 40 3.85 -> 3.67 /
+// 5.09 -> 4.87 ms, 16384 samples 1.45 -> 1.37 / 1.81 -> 1.73 ms.
 // Outputs past the bond dimension are never used.
 template <int SB, int XB>
 __device__ __forceinline__ void f32_contract(const float* M, int P, int dK, const float* X, int g, int sg,
@@ -137,10 +142,26 @@ __device__ __forceinline__ void f32_contract(const float* M, int P, int dK, cons
   auto products = [&](const float (&xk)[SB], const float (&mk)[2 * XB]) {
 #pragma unroll
     for (int j = 0; j < XB; ++j)
+      if constexpr (SB < 8 && SB < 2 * XB) {
+        const float2 mm = make_float2(mk[2 * j], mk[2 * j + 1]);
 #pragma unroll
-      for (int b = 0; b < SB; ++b) {
-        acc[0][j][b] = fmaf(mk[2 * j], xk[b], acc[0][j][b]);
-        acc[1][j][b] = fmaf(mk[2 * j + 1], xk[b], acc[1][j][b]);
+        for (int b = 0; b < SB; ++b) {
+          const float2 r = umma::f2_fma(mm, make_float2(xk[b], xk[b]), make_float2(acc[0][j][b], acc[1][j][b]));
+          acc[0][j][b] = r.x; acc[1][j][b] = r.y;
+        }
+      } else if constexpr (SB > 1) {
+        const float2 m0 = make_float2(mk[2 * j], mk[2 * j]), m1 = make_float2(mk[2 * j + 1], mk[2 * j + 1]);
+#pragma unroll
+        for (int b = 0; b < SB; b += 2) {
+          const float2 x2 = make_float2(xk[b], xk[b + 1]);
+          const float2 r0 = umma::f2_fma(m0, x2, make_float2(acc[0][j][b], acc[0][j][b + 1]));
+          const float2 r1 = umma::f2_fma(m1, x2, make_float2(acc[1][j][b], acc[1][j][b + 1]));
+          acc[0][j][b] = r0.x; acc[0][j][b + 1] = r0.y;
+          acc[1][j][b] = r1.x; acc[1][j][b + 1] = r1.y;
+        }
+      } else {
+        acc[0][j][0] = fmaf(mk[2 * j], xk[0], acc[0][j][0]);
+        acc[1][j][0] = fmaf(mk[2 * j + 1], xk[0], acc[1][j][0]);
       }
   };
   if constexpr (XB > 8) {      // no registers for a second set of operands
