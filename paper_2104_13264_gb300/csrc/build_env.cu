@@ -414,9 +414,91 @@ __device__ inline void tournament(int t, int i, int N, int& p, int& q) {
   }
 }
 
+constexpr double kJacobiTol = 1e-13;
+constexpr int kJacobiSweeps = 40;
+constexpr double kNullRel = 1e-13;
+constexpr int kDotLanes = kBuildThreads / 64;      // partial sums of a row product
+
+// FP64 values as integers.  The FP64 pipe takes one warp instruction per 19 cycles and SM and
+// holds a warp for 64, so comparisons and halvings around the rotations run on the integer pipe;
+// every result is the bits of the FP64 instruction's.
+__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+// largest of the non-negative or NaN d[0 .. m-1], NaN skipped
+__device__ __forceinline__ double max_nonneg(const double* d, int m) {
+  long long mx = 0;
+  for (int i = 0; i < m; ++i) {
+    const long long v = dbits(d[i]);
+    if (v <= 0x7ff0000000000000ll && v > mx) mx = v;
+  }
+  return __longlong_as_double(mx);
+}
+// Lanes per pair: at least the kDotLanes that hold the partial sums of the row product; with few
+// pairs more, which share the rotation, as long as the CTA's active warps stay at four
+// (`threads` active threads for these pairs): more of them would only repeat the scalar work.
+__device__ __forceinline__ int pair_lanes_log2(int npairs, int threads) {
+  int lw = 31 - __clz(kDotLanes);
+  while (lw < 5 && (npairs << (lw + 1)) <= threads) ++lw;
+  return lw;
+}
+
+// Pair `grp` of a round on 2^lw lanes (lane gl): rotates rows p and q of J where
+// |gamma| > tol sqrt(alpha beta).  All lanes of a warp call it.  Returns whether it rotated.
+// Measured against four lanes for every pair and FP64 comparisons: 16 x 48, chi 32 without fields
+// 575 -> 516 ms; 16 x 24, chi 16 with fields 200 -> 151 ms (the extra lanes alone: 181 -> 155);
+// the extra lanes up to eight warps: 165 ms.
+__device__ __forceinline__ bool jacobi_pair(double* J, double* d, int n, int ld, int p, int q, bool live, int gl, int lw,
+                                            double dnull) {
+  const int L = 1 << lw;
+  double* rp = J + (size_t)(live ? p : 0) * ld;
+  double* rq = J + (size_t)(live ? q : 0) * ld;
+  double al = 0.0, be = 0.0, ga = 0.0;
+  if (live) {
+    al = d[p];
+    be = d[q];
+    if (gl < kDotLanes)
+      for (int x = gl; x < n; x += kDotLanes) ga += rp[x] * rq[x];
+  }
+#pragma unroll
+  for (int o = 1; o < kDotLanes; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+  if (L > kDotLanes) ga = __shfl_sync(0xffffffffu, ga, 0, L);
+  // al, be > dnull >= 0 and ga^2 > tol^2 al be (a NaN on either side: no)
+  const long long nul = dbits(dnull), inf = 0x7ff0000000000000ll;
+  if (!live || dbits(al) <= nul || dbits(be) <= nul) return false;
+  const unsigned long long g2 = dbits(ga * ga), lim = dbits(kJacobiTol * kJacobiTol * al * be);
+  if (g2 <= lim || g2 > (unsigned long long)inf) return false;
+  // tangent of the rotation angle in FP32 (its accuracy only sets the convergence rate); cos
+  // from it by two FP64 Newton steps for 1/sqrt, so the applied rotation is orthogonal to FP64
+  // rounding whatever t is
+  const double diff = be - al;
+  float zeta = (float)diff / (2.0f * (float)ga);
+  if (!isfinite(zeta)) zeta = (float)(diff / (2.0 * ga));   // outside FP32 range
+  float tf;
+  if (fabsf(zeta) > 1e18f) tf = 0.5f / zeta;
+  else tf = (zeta >= 0.0f ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
+  const double tt = (double)tf;
+  const double x = fma(tt, tt, 1.0);                                               // [1, 2]
+  const double hx = __hiloint2double((__double2hiint(x) - 0x100000) ^ 0x80000000, __double2loint(x));   // -x / 2
+  double cs = (double)rsqrtf((float)x);
+  cs = cs * fma(hx, cs * cs, 1.5);
+  cs = cs * fma(hx, cs * cs, 1.5);
+  const double sn = cs * tt;
+  for (int xx = gl; xx < n; xx += L) {
+    const double u = rp[xx], v = rq[xx];
+    rp[xx] = cs * u - sn * v;
+    rq[xx] = sn * u + cs * v;
+  }
+  if (gl < 2) {
+    // alpha' on lane 0, beta' on lane 1
+    const double t2 = (double)(gl ? 2.0f * tf : -2.0f * tf);
+    const double self = gl ? be : al, other = gl ? al : be;
+    d[gl ? q : p] = cs * cs * fma(tt * tt, other, fma(t2, ga, self));
+  }
+  return true;
+}
+
 // One-sided Jacobi (Hestenes): orthogonalise the m <= 128 rows (length n, stride
-// ld) of J.  Round-robin pairing; a group of L lanes owns one pair, with L chosen
-// so that all m/2 pairs of a round run at once on the CTA's threads.  Squared row
+// ld) of J.  Round-robin pairing; a group of lanes owns one pair, so that all m/2
+// pairs of a round run at once on the CTA's threads.  Squared row
 // norms d[] are maintained through the exact update alpha' = alpha - t gamma,
 // beta' = beta + t gamma and recomputed at the start of every sweep.  A pair is
 // rotated while |gamma| > tol sqrt(alpha beta), tol = 1e-13 (above the rounding
@@ -425,17 +507,12 @@ __device__ inline void tournament(int t, int i, int N, int& p, int& q) {
 // and are left out of the rotations (callers treat them as zero rows).  Returns
 // false when the last of kJacobiSweeps sweeps still rotated (not converged); the
 // value is the same on every thread.
-constexpr double kJacobiTol = 1e-13;
-constexpr int kJacobiSweeps = 40;
-constexpr double kNullRel = 1e-13;
-
 __device__ bool jacobi_rows(double* J, int m, int n, int ld, double* d, int* flag) {
   const int N = m + (m & 1);
   const int npairs = N / 2;
-  // blockDim.x / 64 lanes per pair (a power of two): all m/2 <= 64 pairs of a round
-  // at once; the per-pair scalar work is repeated on every lane of a group
-  const int L = blockDim.x / 64;
-  const int grp = threadIdx.x / L, gl = threadIdx.x % L;
+  const int lw = pair_lanes_log2(npairs, 128);
+  const int grp = threadIdx.x >> lw, gl = threadIdx.x & ((1 << lw) - 1);
+  const bool warp_live = ((threadIdx.x & ~31) >> lw) < npairs;
   for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
       double s = 0.0;
@@ -444,53 +521,14 @@ __device__ bool jacobi_rows(double* J, int m, int n, int ld, double* d, int* fla
     }
     if (threadIdx.x == 0) flag[0] = 0;
     __syncthreads();
-    double dmax = 0.0;
-    for (int i = 0; i < m; ++i) dmax = fmax(dmax, d[i]);
-    const double dnull = kNullRel * kNullRel * dmax;
+    const double dnull = kNullRel * kNullRel * max_nonneg(d, m);
+    __syncthreads();      // every warp has read d
     for (int t = 0; t < N - 1; ++t) {
-      {
-        // every lane runs the group shuffles below (full-warp masks); groups beyond
-        // the round's pairs only contribute zeros.  m <= 128 gives at most 64 pairs,
-        // one per group of lanes.
+      if (warp_live) {
         int p = m, q = m;
         if (grp < npairs) tournament(t, grp, N, p, q);
-        const bool live = p < m && q < m;
-        double ga = 0.0;
-        double* rp = J + (size_t)(live ? p : 0) * ld;
-        double* rq = J + (size_t)(live ? q : 0) * ld;
-        if (live)
-          for (int x = gl; x < n; x += L) ga += rp[x] * rq[x];
-        for (int o = 1; o < L; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        if (live) {
-          const double al = d[p], be = d[q];
-          if (ga != 0.0 && al > dnull && be > dnull && ga * ga > kJacobiTol * kJacobiTol * al * be) {
-            // tangent of the rotation angle in FP32 (its accuracy only sets the
-            // convergence rate); cos from it by two FP64 Newton steps for 1/sqrt, so the
-            // applied rotation is orthogonal to FP64 rounding whatever t is
-            float zeta = (float)(be - al) / (2.0f * (float)ga);
-            if (!isfinite(zeta)) zeta = (float)((be - al) / (2.0 * ga));   // outside FP32 range
-            float tf;
-            if (fabsf(zeta) > 1e18f) tf = 0.5f / zeta;
-            else tf = (zeta >= 0.0f ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
-            const double tt = (double)tf;
-            const double x = fma(tt, tt, 1.0);
-            double cs = (double)rsqrtf((float)x);
-            cs = cs * fma(-0.5 * x, cs * cs, 1.5);
-            cs = cs * fma(-0.5 * x, cs * cs, 1.5);
-            const double sn = cs * tt;
-            for (int xx = gl; xx < n; xx += L) {
-              const double u = rp[xx], v = rq[xx];
-              rp[xx] = cs * u - sn * v;
-              rq[xx] = sn * u + cs * v;
-            }
-            if (gl == 0) {
-              const double c2 = cs * cs;
-              d[p] = c2 * fma(tt * tt, be, fma(-2.0 * tt, ga, al));
-              d[q] = c2 * fma(tt * tt, al, fma(2.0 * tt, ga, be));
-              flag[0] = 1;
-            }
-          }
-        }
+        if (jacobi_pair(J, d, n, ld, p, q, p < m && q < m, gl, lw, dnull) && gl == 0) flag[0] = 1;
+        __syncwarp();
       }
       __syncthreads();
     }
@@ -1185,8 +1223,7 @@ __device__ inline int z2_col(int s, int j, int Dr, int er) {
 
 // Both parity sectors of a site at once: the first half of the threads orthogonalises
 // the m0 rows of J0, the second half the m1 rows of J1 (m0, m1 <= 64; same n, ld), each
-// with the rounds, tolerances and arithmetic of jacobi_rows (blockDim.x / 64 lanes per
-// pair, a power of two).  Sweeps continue until neither
+// with the rounds, tolerances and arithmetic of jacobi_rows.  Sweeps continue until neither
 // sector rotates; a converged sector's extra sweep rotates nothing.
 __device__ bool jacobi_rows2(double* J0, int m0, double* J1, int m1, int n, int ld, double* d0, double* d1,
                              int* flag) {
@@ -1199,8 +1236,9 @@ __device__ bool jacobi_rows2(double* J0, int m0, double* J1, int m1, int n, int 
   const int N = m + (m & 1);
   const int npairs = N / 2;
   const int Nmax = max(m0 + (m0 & 1), m1 + (m1 & 1));
-  const int L = half / 32;                   // lanes per pair: all 32 pairs of a round at once
-  const int grp = lt / L, gl = lt % L;
+  const int lw = pair_lanes_log2(Nmax / 2, 64);
+  const int grp = lt >> lw, gl = lt & ((1 << lw) - 1);
+  const bool warp_live = ((lt & ~31) >> lw) < npairs;
   for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
     for (int i = lt; i < m; i += half) {
       double s = 0.0;
@@ -1212,48 +1250,14 @@ __device__ bool jacobi_rows2(double* J0, int m0, double* J1, int m1, int n, int 
       flag[2] = 0;
     }
     __syncthreads();
-    double dmax = 0.0;
-    for (int i = 0; i < m; ++i) dmax = fmax(dmax, d[i]);
-    const double dnull = kNullRel * kNullRel * dmax;
+    const double dnull = kNullRel * kNullRel * max_nonneg(d, m);
+    __syncthreads();      // every warp has read d
     for (int t = 0; t < Nmax - 1; ++t) {
-      {
-        // groups beyond this sector's pairs (or rounds) only contribute zeros to the shuffles
+      if (warp_live && t < N - 1) {
         int p = m, q = m;
-        if (grp < npairs && t < N - 1) tournament(t, grp, N, p, q);
-        const bool live = p < m && q < m;
-        double ga = 0.0;
-        double* rp = J + (size_t)(live ? p : 0) * ld;
-        double* rq = J + (size_t)(live ? q : 0) * ld;
-        if (live)
-          for (int x = gl; x < n; x += L) ga += rp[x] * rq[x];
-        for (int o = 1; o < L; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        if (live) {
-          const double al = d[p], be = d[q];
-          if (ga != 0.0 && al > dnull && be > dnull && ga * ga > kJacobiTol * kJacobiTol * al * be) {
-            float zeta = (float)(be - al) / (2.0f * (float)ga);
-            if (!isfinite(zeta)) zeta = (float)((be - al) / (2.0 * ga));
-            float tf;
-            if (fabsf(zeta) > 1e18f) tf = 0.5f / zeta;
-            else tf = (zeta >= 0.0f ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
-            const double tt = (double)tf;
-            const double x = fma(tt, tt, 1.0);
-            double cs = (double)rsqrtf((float)x);
-            cs = cs * fma(-0.5 * x, cs * cs, 1.5);
-            cs = cs * fma(-0.5 * x, cs * cs, 1.5);
-            const double sn = cs * tt;
-            for (int xx = gl; xx < n; xx += L) {
-              const double u = rp[xx], v = rq[xx];
-              rp[xx] = cs * u - sn * v;
-              rq[xx] = sn * u + cs * v;
-            }
-            if (gl == 0) {
-              const double c2 = cs * cs;
-              d[p] = c2 * fma(tt * tt, be, fma(-2.0 * tt, ga, al));
-              d[q] = c2 * fma(tt * tt, al, fma(2.0 * tt, ga, be));
-              flag[2 * sec] = 1;
-            }
-          }
-        }
+        if (grp < npairs) tournament(t, grp, N, p, q);
+        if (jacobi_pair(J, d, n, ld, p, q, p < m && q < m, gl, lw, dnull) && gl == 0) flag[2 * sec] = 1;
+        __syncwarp();
       }
       __syncthreads();
     }
