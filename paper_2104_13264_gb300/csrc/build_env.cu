@@ -197,69 +197,156 @@ __device__ void apply_row_mpo(const BuildArgs& a, Shared& sh, int r) {
 }
 
 // ---------------------------------------------------------------------------
-// Householder QR of a column-major m x n matrix A (lda = m) in shared memory.
-// On exit: R (k x n, k = min(m, n)) in Rout (row-major, ld n), Q (m x k) in Q
-// (column-major, ld m).  Reflector j is stored in A[j*m + j .. ], tau[j].
+// Householder QR of a column-major m x n matrix A (lda = m <= 128) in shared memory by a team of
+// `nw` >= 2 warps (w: the warp's number in its team; barrier `bar` of the team's threads).
+// On exit: R (k x n, k = min(m, n)) in Rout (row-major, ld n), Q (m x k) in A (column-major,
+// ld m).
+//
+// What bounds it: FP64 issue (one warp instruction per 19 cycles and SM) and the chain norm ->
+// square root -> division of one reflector, about 3000 cycles.  So the two independent blocks of
+// a site run at once on half the warps each; warp 0 of a team updates the next column first and
+// makes its reflector while the others update the rest; and up to four columns of a warp share
+// the reduction of their products (6 additions instead of 20, each pair and order as in
+// warp_sum).  Q is formed in place, which lets both blocks fit.
+// Measured against one block after the other on all warps, a reduction per column: 16 x 48, chi 32
+// without fields 516 -> 451 ms; 16 x 24, chi 16 with fields 151 -> 140 ms.
 // ---------------------------------------------------------------------------
-__device__ void householder_qr(double* A, int m, int n, double* Q, double* Rout, double* tau,
-                               double* diag) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int k = min(m, n);
-  for (int j = 0; j < k; ++j) {
-    if (w == 0) {
-      double s = 0.0;
-      for (int i = j + lane; i < m; i += 32) s += A[j * m + i] * A[j * m + i];
-      s = warp_sum(s);
-      if (lane == 0) {
-        const double x0 = A[j * m + j];
-        const double nrm = sqrt(s);
-        if (nrm == 0.0) {
-          tau[j] = 0.0;
-          diag[j] = 0.0;
-        } else {
-          const double alpha = (x0 > 0.0) ? -nrm : nrm;
-          const double v0 = x0 - alpha;
-          A[j * m + j] = v0;
-          tau[j] = -1.0 / (alpha * v0);
-          diag[j] = alpha;
-        }
-      }
+__device__ __forceinline__ void team_sync(int bar, int nw) {
+  asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(32 * nw) : "memory");
+}
+
+// warp_sum of NC values at once: afterwards lanes 8 g .. 8 g + 7 hold the sum of value
+// g (NC = 4), (g >> 1) (NC = 2) or 0 (NC = 1)
+template <int NC>
+__device__ __forceinline__ double warp_sum_packed(const double (&v)[NC]) {
+  const unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  double r;
+  if constexpr (NC == 1) {
+    r = v[0] + __shfl_xor_sync(kFull, v[0], 16);
+    r += __shfl_xor_sync(kFull, r, 8);
+  } else {
+    const bool h = lane & 16;
+    if constexpr (NC == 2) {
+      r = (h ? v[1] : v[0]) + __shfl_xor_sync(kFull, h ? v[0] : v[1], 16);
+      r += __shfl_xor_sync(kFull, r, 8);
+    } else {
+      const double r0 = (h ? v[2] : v[0]) + __shfl_xor_sync(kFull, h ? v[0] : v[2], 16);
+      const double r1 = (h ? v[3] : v[1]) + __shfl_xor_sync(kFull, h ? v[1] : v[3], 16);
+      const bool g = lane & 8;
+      r = (g ? r1 : r0) + __shfl_xor_sync(kFull, g ? r0 : r1, 8);
     }
-    __syncthreads();
-    const double t = tau[j];
-    if (t != 0.0) {
-      for (int l = j + 1 + w; l < n; l += kWarps) {
-        double d = 0.0;
-        for (int i = j + lane; i < m; i += 32) d += A[j * m + i] * A[l * m + i];
-        d = warp_sum(d) * t;
-        for (int i = j + lane; i < m; i += 32) A[l * m + i] -= d * A[j * m + i];
-      }
-    }
-    __syncthreads();
   }
-  // R
-  for (int idx = threadIdx.x; idx < k * n; idx += blockDim.x) {
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+  return r;
+}
+
+// Reflector v (rows j .. m-1, factor t) applied to the columns at c, c + step, ... (NC of them)
+template <int NC>
+__device__ __forceinline__ void reflect_columns(const double* v, double t, double* c, size_t step, int j, int m) {
+  const int lane = threadIdx.x & 31;
+  double d[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) d[q] = 0.0;
+  for (int i = j + lane; i < m; i += 32) {
+    const double x = v[i];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) d[q] += x * c[q * step + i];
+  }
+  const double s = warp_sum_packed<NC>(d) * t;
+#pragma unroll
+  for (int q = 0; q < NC; ++q) d[q] = __shfl_sync(0xffffffffu, s, NC == 4 ? 8 * q : 16 * q);
+  for (int i = j + lane; i < m; i += 32) {
+    const double x = v[i];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) c[q * step + i] -= d[q] * x;
+  }
+}
+
+// Columns l0, l0 + step, ... < n of A
+__device__ __forceinline__ void reflect(const double* v, double t, double* A, int l0, int step, int n, int j, int m) {
+  const size_t cs = (size_t)step * m;
+  int l = l0;
+  for (; l + 2 * step < n; l += 4 * step) {
+    if (l + 3 * step < n) reflect_columns<4>(v, t, A + (size_t)l * m, cs, j, m);
+    else {
+      reflect_columns<2>(v, t, A + (size_t)l * m, cs, j, m);
+      reflect_columns<1>(v, t, A + (size_t)(l + 2 * step) * m, cs, j, m);
+    }
+  }
+  if (l + step < n) reflect_columns<2>(v, t, A + (size_t)l * m, cs, j, m);
+  else if (l < n) reflect_columns<1>(v, t, A + (size_t)l * m, cs, j, m);
+}
+
+// Reflector j from column j (one warp): v_0 in place, tau[j], diag[j]
+__device__ __forceinline__ void make_reflector(double* A, int m, int j, double* tau, double* diag) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int i = j + lane; i < m; i += 32) s += A[j * m + i] * A[j * m + i];
+  s = warp_sum(s);
+  if (lane == 0) {
+    const double x0 = A[j * m + j];
+    const double nrm = sqrt(s);
+    if (nrm == 0.0) {
+      tau[j] = 0.0;
+      diag[j] = 0.0;
+    } else {
+      const double alpha = (x0 > 0.0) ? -nrm : nrm;
+      const double v0 = x0 - alpha;
+      A[j * m + j] = v0;
+      tau[j] = -1.0 / (alpha * v0);
+      diag[j] = alpha;
+    }
+  }
+}
+
+__device__ void householder_qr(double* A, int m, int n, double* Rout, double* tau, double* diag, int w, int nw,
+                               int bar) {
+  const int lane = threadIdx.x & 31, tid = 32 * w + lane;
+  const int k = min(m, n);
+  if (w == 0) make_reflector(A, m, 0, tau, diag);
+  team_sync(bar, nw);
+  for (int j = 0; j < k; ++j) {
+    const double t = tau[j];
+    const double* v = A + (size_t)j * m;
+    if (w == 0) {
+      if (t != 0.0 && j + 1 < n) reflect_columns<1>(v, t, A + (size_t)(j + 1) * m, 0, j, m);
+      __syncwarp();
+      if (j + 1 < k) make_reflector(A, m, j + 1, tau, diag);
+    } else if (t != 0.0) {
+      reflect(v, t, A, j + 1 + w, nw - 1, n, j, m);
+    }
+    team_sync(bar, nw);
+  }
+  // R, and the rows above the diagonal cleared
+  for (int idx = tid; idx < k * n; idx += 32 * nw) {
     const int j = idx / n, l = idx % n;
     Rout[idx] = (l < j) ? 0.0 : (l == j ? diag[j] : A[l * m + j]);
+    if (l > j) A[l * m + j] = 0.0;
   }
-  // Q = H_0 ... H_{k-1} [I_k; 0]
-  for (int idx = threadIdx.x; idx < m * k; idx += blockDim.x) {
-    const int l = idx / m, i = idx % m;
-    Q[idx] = (i == l) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  for (int j = k - 1; j >= 0; --j) {
+  team_sync(bar, nw);
+  // Q = H_0 ... H_{k-1} [I_k; 0]: column j turns from the reflector to H_j e_j once the columns
+  // behind it have been reflected, one step later, by the warp that updates it next
+  auto finish = [&](int j) {
     const double t = tau[j];
-    if (t != 0.0) {
-      for (int l = j + w; l < k; l += kWarps) {
-        double d = 0.0;
-        for (int i = j + lane; i < m; i += 32) d += A[j * m + i] * Q[l * m + i];
-        d = warp_sum(d) * t;
-        for (int i = j + lane; i < m; i += 32) Q[l * m + i] -= d * A[j * m + i];
-      }
+    double* c = A + (size_t)j * m;
+    const double v0 = c[j], d = v0 * t;
+    __syncwarp();
+    for (int i = j + lane; i < m; i += 32) {
+      const double e = i == j ? 1.0 : 0.0;
+      c[i] = t != 0.0 ? fma(-d, c[i], e) : e;
     }
-    __syncthreads();
+    __syncwarp();
+  };
+  for (int j = k - 1; j >= 0; --j) {
+    if (w == 0 && j + 1 < k) finish(j + 1);
+    const double t = tau[j];
+    if (t != 0.0) reflect(A + (size_t)j * m, t, A, j + 1 + w, nw, k, j, m);
+    team_sync(bar, nw);
   }
+  if (w == 0) finish(0);
+  team_sync(bar, nw);
 }
 
 // ---------------------------------------------------------------------------
@@ -268,14 +355,13 @@ __device__ void householder_qr(double* A, int m, int n, double* Q, double* Rout,
 // Bond basis: the upper factor T mixes the physical index, so the site tensors lose the
 // copy structure (physical spin == right horizontal copy) that qr_sweep factors block
 // by block.  Here each site is one (2 m) x Dr matrix, rows (left, physical), and its QR
-// gives a new bond of min(2 m, Dr).  Dims stay <= 2 max_bond <= P, so A and Q fit in
-// 2 P^2 doubles each and R in P^2.
+// gives a new bond of min(2 m, Dr).  Dims stay <= 2 max_bond <= P, so A fits in 2 P^2
+// doubles and R in P^2.
 __device__ double qr_sweep_dense(const BuildArgs& a, Shared& sh) {
   const int Lx = a.Lx, P = a.P;
   const size_t slot_sz = (size_t)8 * P * P;
   double logs = 0.0;
   double* A = sh.W;
-  double* Q = sh.W + 2 * P * P;
   double* Rb = sh.W + 4 * P * P;
   double* tau = sh.W + 6 * P * P;
   double* diag = tau + P;
@@ -290,11 +376,10 @@ __device__ double qr_sweep_dense(const BuildArgs& a, Shared& sh) {
       A[idx] = X[(size_t)q * Dr + l];
     }
     __syncthreads();
-    householder_qr(A, M, Dr, Q, Rb, tau, diag);
-    __syncthreads();
+    householder_qr(A, M, Dr, Rb, tau, diag, threadIdx.x >> 5, kWarps, 1);
     for (int idx = threadIdx.x; idx < M * k; idx += blockDim.x) {
       const int j = idx / M, q = idx % M;
-      Tn[(size_t)q * k + j] = Q[j * M + q];
+      Tn[(size_t)q * k + j] = A[j * M + q];
     }
     double mx = 0.0;
     for (int idx = threadIdx.x; idx < k * Dr; idx += blockDim.x) mx = fmax(mx, fabs(Rb[idx]));
@@ -336,10 +421,12 @@ __device__ double qr_sweep(const BuildArgs& a, Shared& sh) {
   const int Lx = a.Lx, P = a.P;
   const size_t slot_sz = (size_t)8 * P * P;
   double logs = 0.0;
-  double* A = sh.W;
-  double* Q = sh.W + 2 * P * P;
-  double* Rb = sh.W + 4 * P * P;   // R_0 at Rb, R_1 at Rb + P*P
-  double* tau = sh.W + 6 * P * P;
+  // half the CTA's warps per spin block: A at W + 2 P^2 sp, R at W + (4 + sp) P^2
+  constexpr int kTeam = kWarps / 2;
+  const int sp = threadIdx.x / (32 * kTeam), lt = threadIdx.x % (32 * kTeam);
+  double* A = sh.W + (size_t)sp * 2 * P * P;
+  double* Rb = sh.W + 4 * P * P;
+  double* tau = sh.W + 6 * P * P + (size_t)sp * 2 * P;
   double* diag = tau + P;
   for (int c = 0; c < Lx - 1; ++c) {
     const int m = sh.dl[c];
@@ -348,22 +435,19 @@ __device__ double qr_sweep(const BuildArgs& a, Shared& sh) {
     const int k = min(m, nb);
     const double* X = a.work + (size_t)sh.slot[c] * slot_sz;
     double* Tn = a.work + (size_t)sh.slot[Lx] * slot_sz;   // new site c: [m][2][2k]
-    for (int sp = 0; sp < 2; ++sp) {
-      for (int idx = threadIdx.x; idx < m * nb; idx += blockDim.x) {
-        const int l = idx / m, i = idx % m;   // column-major A[l*m + i]
-        A[idx] = X[((size_t)i * 2 + sp) * Dr + l * 2 + sp];
-      }
-      __syncthreads();
-      householder_qr(A, m, nb, Q, Rb + sp * P * P, tau, diag);
-      __syncthreads();
-      // new tensor entries (i, s, (j, s')) with s == s' == sp
-      for (int idx = threadIdx.x; idx < m * k; idx += blockDim.x) {
-        const int j = idx / m, i = idx % m;
-        Tn[((size_t)i * 2 + sp) * (2 * k) + j * 2 + sp] = Q[j * m + i];
-        Tn[((size_t)i * 2 + sp) * (2 * k) + j * 2 + (1 - sp)] = 0.0;
-      }
-      __syncthreads();
+    for (int idx = lt; idx < m * nb; idx += 32 * kTeam) {
+      const int l = idx / m, i = idx % m;   // column-major A[l*m + i]
+      A[idx] = X[((size_t)i * 2 + sp) * Dr + l * 2 + sp];
     }
+    team_sync(1 + sp, kTeam);
+    householder_qr(A, m, nb, Rb + sp * P * P, tau, diag, lt >> 5, kTeam, 1 + sp);
+    // new tensor entries (i, s, (j, s')) with s == s' == sp
+    for (int idx = lt; idx < m * k; idx += 32 * kTeam) {
+      const int j = idx / m, i = idx % m;
+      Tn[((size_t)i * 2 + sp) * (2 * k) + j * 2 + sp] = A[j * m + i];
+      Tn[((size_t)i * 2 + sp) * (2 * k) + j * 2 + (1 - sp)] = 0.0;
+    }
+    __syncthreads();
     // scale of R
     double mx = 0.0;
     for (int idx = threadIdx.x; idx < k * nb; idx += blockDim.x)
@@ -1144,10 +1228,12 @@ __device__ double qr_sweep_z2(const BuildArgs& a, ShZ2& sh) {
   const int Lx = a.Lx, P = a.P;
   const size_t slot_sz = (size_t)8 * P * P;
   double logs = 0.0;
-  double* A = sh.W;
-  double* Q = sh.W + 2 * P * P;
+  // half the CTA's warps per parity sector: A at W + 2 P^2 s, R at W + (4 + s) P^2
+  constexpr int kTeam = kWarps / 2;
+  const int s = threadIdx.x / (32 * kTeam), lt = threadIdx.x % (32 * kTeam);
+  double* A = sh.W + (size_t)s * 2 * P * P;
   double* Rb = sh.W + 4 * P * P;
-  double* tau = sh.W + 6 * P * P;
+  double* tau = sh.W + 6 * P * P + (size_t)s * 2 * P;
   double* diag = tau + P;
   for (int c = 0; c < Lx - 1; ++c) {
     const int Dl = sh.bdim[c], el = sh.bev[c], Dr = sh.bdim[c + 1], er = sh.bev[c + 1];
@@ -1157,24 +1243,23 @@ __device__ double qr_sweep_z2(const BuildArgs& a, ShZ2& sh) {
     double* Tn = a.work + (size_t)sh.slot[Lx] * slot_sz;   // new site c: [Dl][2][K]
     for (int idx = threadIdx.x; idx < Dl * 2 * K; idx += blockDim.x) Tn[idx] = 0.0;
     __syncthreads();
-    for (int s = 0; s < 2; ++s) {
-      const int ns = s ? n1 : n0, col0 = s ? er : 0, ks = s ? k1 : k0, j0 = s ? k0 : 0;
-      if (ns == 0) continue;
-      for (int idx = threadIdx.x; idx < Dl * ns; idx += blockDim.x) {
+    const int ns = s ? n1 : n0, ks = s ? k1 : k0;
+    if (ns > 0) {
+      const int col0 = s ? er : 0, j0 = s ? k0 : 0;
+      for (int idx = lt; idx < Dl * ns; idx += 32 * kTeam) {
         const int j = idx / Dl, l = idx % Dl;
         const int tl = s ^ (l >= el ? 1 : 0);
         A[idx] = X[((size_t)l * 2 + tl) * Dr + col0 + j];
       }
-      __syncthreads();
-      householder_qr(A, Dl, ns, Q, Rb + s * P * P, tau, diag);
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < Dl * ks; idx += blockDim.x) {
+      team_sync(1 + s, kTeam);
+      householder_qr(A, Dl, ns, Rb + s * P * P, tau, diag, lt >> 5, kTeam, 1 + s);
+      for (int idx = lt; idx < Dl * ks; idx += 32 * kTeam) {
         const int j = idx / Dl, l = idx % Dl;
         const int tl = s ^ (l >= el ? 1 : 0);
-        Tn[((size_t)l * 2 + tl) * K + j0 + j] = Q[j * Dl + l];
+        Tn[((size_t)l * 2 + tl) * K + j0 + j] = A[j * Dl + l];
       }
-      __syncthreads();
     }
+    __syncthreads();
     double mx = 0.0;
     for (int idx = threadIdx.x; idx < k0 * n0; idx += blockDim.x) mx = fmax(mx, fabs(Rb[idx]));
     for (int idx = threadIdx.x; idx < k1 * n1; idx += blockDim.x) mx = fmax(mx, fabs(Rb[P * P + idx]));
