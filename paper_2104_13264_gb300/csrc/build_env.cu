@@ -1,6 +1,7 @@
 // FP64 boundary-MPS builder (App. A, eq. braket-top-tm-bot; "successive SVD").
 //
-// One CTA builds every row environment of one instance, bottom-up:
+// One CTA builds every row environment of one instance (two, a parity sector each, where all
+// fields are zero and the bonds are large), bottom-up:
 //   env_{Ly-1} = exact weight of row Ly-1;  env_r = T_chi[ D_r H_r V_r env_{r+1} ].
 // Per row:
 //   1. MPO application (V_r vertical bonds, D_r fields, H_r horizontal bonds as a
@@ -17,6 +18,7 @@
 //      the way is accumulated in log_scale[r].
 // Working tensors live in global scratch slots (L2 resident); the linear algebra
 // of one site runs in shared memory.  All arithmetic is FP64.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <new>
@@ -1224,12 +1226,52 @@ __device__ void apply_row_mpo_z2(const BuildArgs& a, ShZ2& sh, int r) {
   __syncthreads();
 }
 
+// A cluster of two CTAs: the main one builds, the other takes parity sector 1 of each QR and
+// each Jacobi iteration (the sectors are independent in both).  A command goes through flag[4 .. 7]
+// of the main CTA's shared memory between two cluster barriers; the tensors are read from the
+// work slots, the results go back to the main CTA's shared memory.
+//   flag[4]: kCmdExit, kCmdQr or kCmdJacobi | el << 8 | Dl << 16; flag[5]: Dr | er << 16;
+//   flag[6]: slot read | slot written << 16; flag[7]: the Jacobi iteration converged
+constexpr int kCmdExit = 0, kCmdQr = 1, kCmdJacobi = 2;
+
+__device__ __forceinline__ void send_command(ShZ2& sh, int cmd, int el, int Dl, int Dr, int er, int src, int dst) {
+  if (threadIdx.x == 0) {
+    sh.flag[4] = cmd | el << 8 | Dl << 16;
+    sh.flag[5] = Dr | er << 16;
+    sh.flag[6] = src | dst << 16;
+  }
+  cooperative_groups::this_cluster().sync();
+}
+
+// QR of parity sector s of a site (right index in the sector) by a team of nw warps; k0, K: new
+// bond, its even part; A, R, tau, diag: the team's work areas
+__device__ void qr_block_z2(const double* X, double* Tn, int Dl, int el, int Dr, int er, int s, double* A, double* R,
+                            double* tau, double* diag, int lt, int nw, int bar) {
+  const int k0 = min(Dl, er), k1 = min(Dl, Dr - er), K = k0 + k1;
+  const int ns = s ? Dr - er : er, ks = s ? k1 : k0, col0 = s ? er : 0, j0 = s ? k0 : 0;
+  if (ns == 0) return;
+  for (int idx = lt; idx < Dl * ns; idx += 32 * nw) {
+    const int j = idx / Dl, l = idx % Dl;
+    const int tl = s ^ (l >= el ? 1 : 0);
+    A[idx] = X[((size_t)l * 2 + tl) * Dr + col0 + j];
+  }
+  team_sync(bar, nw);
+  householder_qr(A, Dl, ns, R, tau, diag, lt >> 5, nw, bar);
+  for (int idx = lt; idx < Dl * ks; idx += 32 * nw) {
+    const int j = idx / Dl, l = idx % Dl;
+    const int tl = s ^ (l >= el ? 1 : 0);
+    Tn[((size_t)l * 2 + tl) * K + j0 + j] = A[j * Dl + l];
+  }
+}
+
+template <bool PAIR>
 __device__ double qr_sweep_z2(const BuildArgs& a, ShZ2& sh) {
   const int Lx = a.Lx, P = a.P;
   const size_t slot_sz = (size_t)8 * P * P;
   double logs = 0.0;
-  // half the CTA's warps per parity sector: A at W + 2 P^2 s, R at W + (4 + s) P^2
-  constexpr int kTeam = kWarps / 2;
+  // half the CTA's warps per parity sector (PAIR: all of them for sector 0): A at W + 2 P^2 s,
+  // R at W + (4 + s) P^2
+  constexpr int kTeam = PAIR ? kWarps : kWarps / 2;
   const int s = threadIdx.x / (32 * kTeam), lt = threadIdx.x % (32 * kTeam);
   double* A = sh.W + (size_t)s * 2 * P * P;
   double* Rb = sh.W + 4 * P * P;
@@ -1243,23 +1285,10 @@ __device__ double qr_sweep_z2(const BuildArgs& a, ShZ2& sh) {
     double* Tn = a.work + (size_t)sh.slot[Lx] * slot_sz;   // new site c: [Dl][2][K]
     for (int idx = threadIdx.x; idx < Dl * 2 * K; idx += blockDim.x) Tn[idx] = 0.0;
     __syncthreads();
-    const int ns = s ? n1 : n0, ks = s ? k1 : k0;
-    if (ns > 0) {
-      const int col0 = s ? er : 0, j0 = s ? k0 : 0;
-      for (int idx = lt; idx < Dl * ns; idx += 32 * kTeam) {
-        const int j = idx / Dl, l = idx % Dl;
-        const int tl = s ^ (l >= el ? 1 : 0);
-        A[idx] = X[((size_t)l * 2 + tl) * Dr + col0 + j];
-      }
-      team_sync(1 + s, kTeam);
-      householder_qr(A, Dl, ns, Rb + s * P * P, tau, diag, lt >> 5, kTeam, 1 + s);
-      for (int idx = lt; idx < Dl * ks; idx += 32 * kTeam) {
-        const int j = idx / Dl, l = idx % Dl;
-        const int tl = s ^ (l >= el ? 1 : 0);
-        Tn[((size_t)l * 2 + tl) * K + j0 + j] = A[j * Dl + l];
-      }
-    }
-    __syncthreads();
+    if (PAIR) send_command(sh, kCmdQr, el, Dl, Dr, er, sh.slot[c], sh.slot[Lx]);
+    qr_block_z2(X, Tn, Dl, el, Dr, er, s, A, Rb + s * P * P, tau, diag, lt, kTeam, 1 + s);
+    if (PAIR) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
     double mx = 0.0;
     for (int idx = threadIdx.x; idx < k0 * n0; idx += blockDim.x) mx = fmax(mx, fabs(Rb[idx]));
     for (int idx = threadIdx.x; idx < k1 * n1; idx += blockDim.x) mx = fmax(mx, fabs(Rb[P * P + idx]));
@@ -1353,6 +1382,15 @@ __device__ bool jacobi_rows2(double* J0, int m0, double* J1, int m1, int n, int 
   return false;
 }
 
+// Rows i0 .. i1-1 of the site matrix A [Dl][2][Dr], each in its parity block's n = Dr columns
+__device__ __forceinline__ void load_rows_z2(double* J, const double* A, int i0, int i1, int el, int Dr, int er) {
+  for (int idx = threadIdx.x; idx < (i1 - i0) * Dr; idx += blockDim.x) {
+    const int l = i0 + idx / Dr, j = idx % Dr;
+    J[(idx / Dr) * (Dr + 1) + j] = A[(size_t)l * 2 * Dr + z2_col(l >= el ? 1 : 0, j, Dr, er)];   // tau * Dr + x
+  }
+}
+
+template <bool PAIR>
 __device__ double svd_sweep_z2(const BuildArgs& a, ShZ2& sh, int r) {
   const int Lx = a.Lx, P = a.P;
   const size_t slot_sz = (size_t)8 * P * P;
@@ -1371,19 +1409,24 @@ __device__ double svd_sweep_z2(const BuildArgs& a, ShZ2& sh, int r) {
       if (threadIdx.x == 0) set_status(a.status, TNMC_E_NUMERIC);
       return logs;
     }
-    for (int idx = threadIdx.x; idx < Dl * n; idx += blockDim.x) {
-      const int l = idx / n, j = idx % n;
-      const int s = l >= el ? 1 : 0;
-      const int col = z2_col(s, j, Dr, er);     // tau * Dr + x
-      J[l * ld + j] = A[(size_t)l * 2 * Dr + col];
-    }
-    __syncthreads();
     bool converged = true;
-    if (el <= 64 && Dl - el <= 64) {
-      converged = jacobi_rows2(J, el, J + (size_t)el * ld, Dl - el, n, ld, nrm, nrm + el, sh.flag);
+    const bool both = el <= 64 && Dl - el <= 64;
+    if (PAIR && both) {
+      send_command(sh, kCmdJacobi, el, Dl, Dr, er, sh.slot[c], 0);
+      load_rows_z2(J, A, 0, el, el, Dr, er);
+      __syncthreads();
+      converged = jacobi_rows(J, el, n, ld, nrm, sh.flag);
+      cooperative_groups::this_cluster().sync();
+      converged = converged && sh.flag[7];
     } else {
-      if (el > 0) converged = jacobi_rows(J, el, n, ld, nrm, sh.flag);
-      if (Dl - el > 0) converged = jacobi_rows(J + (size_t)el * ld, Dl - el, n, ld, nrm + el, sh.flag) && converged;
+      load_rows_z2(J, A, 0, Dl, el, Dr, er);
+      __syncthreads();
+      if (both) {
+        converged = jacobi_rows2(J, el, J + (size_t)el * ld, Dl - el, n, ld, nrm, nrm + el, sh.flag);
+      } else {
+        if (el > 0) converged = jacobi_rows(J, el, n, ld, nrm, sh.flag);
+        if (Dl - el > 0) converged = jacobi_rows(J + (size_t)el * ld, Dl - el, n, ld, nrm + el, sh.flag) && converged;
+      }
     }
     if (!converged && threadIdx.x == 0) set_status(a.status, TNMC_E_NUMERIC);
     for (int i = w; i < Dl; i += kWarps) {
@@ -1492,7 +1535,7 @@ __device__ double svd_sweep_z2(const BuildArgs& a, ShZ2& sh, int r) {
   return logs;
 }
 
-__device__ void build_env_z2_body(const BuildArgs& a, double* smem) {
+__device__ ShZ2 carve_z2(const BuildArgs& a, double* smem) {
   const int Lx = a.Lx, P = a.P;
   ShZ2 sh;
   sh.W = smem;
@@ -1504,13 +1547,53 @@ __device__ void build_env_z2_body(const BuildArgs& a, double* smem) {
   sh.sel = sh.bev + (Lx + 1);
   sh.sec = sh.sel + 2 * P;
   sh.flag = sh.sec + 2 * P;
+  return sh;
+}
+
+// The second CTA of a pair
+__device__ void build_env_z2_second(const BuildArgs& a, double* smem) {
+  auto cluster = cooperative_groups::this_cluster();
+  const int P = a.P;
+  const size_t slot_sz = (size_t)8 * P * P;
+  ShZ2 sh = carve_z2(a, smem);
+  double* mainW = cluster.map_shared_rank(sh.W, 0);
+  int* mainf = cluster.map_shared_rank(sh.flag, 0);
+  while (true) {
+    cluster.sync();
+    const int cmd = mainf[4] & 0xff, el = (mainf[4] >> 8) & 0xff, Dl = mainf[4] >> 16;
+    const int Dr = mainf[5] & 0xffff, er = mainf[5] >> 16;
+    const double* A = a.work + (size_t)(mainf[6] & 0xffff) * slot_sz;
+    if (cmd == kCmdExit) break;
+    if (cmd == kCmdQr) {
+      double* R = sh.W + 4 * P * P;
+      qr_block_z2(A, a.work + (size_t)(mainf[6] >> 16) * slot_sz, Dl, el, Dr, er, 1, sh.W, R, sh.W + 6 * P * P,
+                  sh.W + 6 * P * P + P, threadIdx.x, kWarps, 1);
+      const int n1 = Dr - er, cnt = min(Dl, n1) * n1;
+      for (int i = threadIdx.x; i < cnt; i += blockDim.x) mainW[5 * P * P + i] = R[i];
+    } else {
+      const int m = Dl - el, ld = Dr + 1;
+      load_rows_z2(sh.W, A, el, Dl, el, Dr, er);
+      __syncthreads();
+      const bool ok = jacobi_rows(sh.W, m, Dr, ld, sh.W + 6 * P * P + 2 * P, sh.flag);
+      for (int i = threadIdx.x; i < m * ld; i += blockDim.x) mainW[el * ld + i] = sh.W[i];
+      if (threadIdx.x == 0) mainf[7] = ok;
+    }
+    cluster.sync();
+  }
+  cluster.sync();
+}
+
+template <bool PAIR>
+__device__ void build_env_z2_body(const BuildArgs& a, double* smem) {
+  const int Lx = a.Lx, P = a.P;
+  ShZ2 sh = carve_z2(a, smem);
   const size_t slot_sz = (size_t)8 * P * P;
   const double isq2 = 0.70710678118654752440;
 
   for (int r = a.Ly - 1; r >= 0; --r) {
     apply_row_mpo_z2(a, sh, r);
-    double logs = qr_sweep_z2(a, sh);
-    logs += svd_sweep_z2(a, sh, r);
+    double logs = qr_sweep_z2<PAIR>(a, sh);
+    logs += svd_sweep_z2<PAIR>(a, sh, r);
     const double* T0 = a.work + (size_t)sh.slot[0] * slot_sz;
     const int cnt = sh.bdim[0] * 2 * sh.bdim[1];
     double sq = 0.0;
@@ -1549,6 +1632,10 @@ __device__ void build_env_z2_body(const BuildArgs& a, double* smem) {
     }
     __syncthreads();
   }
+  if (PAIR) {
+    send_command(sh, kCmdExit, 0, 0, 0, 0, 0, 0);
+    cooperative_groups::this_cluster().sync();      // the second CTA has read the command
+  }
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     double* v = sh.W;
@@ -1586,13 +1673,18 @@ __global__ void __launch_bounds__(kBuildThreads) build_env_kernel(BuildArgs a) {
 }
 __global__ void __launch_bounds__(kBuildThreads) build_env_z2_kernel(BuildArgs a) {
   extern __shared__ double smem[];
-  build_env_z2_body(a, smem);
+  build_env_z2_body<false>(a, smem);
+}
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBuildThreads) build_env_z2_pair_kernel(BuildArgs a) {
+  extern __shared__ double smem[];
+  if (blockIdx.x == 0) build_env_z2_body<true>(a, smem);
+  else build_env_z2_second(a, smem);
 }
 // Many instances in one launch, one CTA each (independent problems).
 __global__ void __launch_bounds__(kBuildThreads) build_env_batched_kernel(const BuildArgs* list) {
   extern __shared__ double smem[];
   const BuildArgs a = list[blockIdx.x];
-  if (a.z2) build_env_z2_body(a, smem);
+  if (a.z2) build_env_z2_body<false>(a, smem);
   else build_env_body(a, smem);
 }
 
@@ -1743,8 +1835,14 @@ tnmc_status tnmc_launch_build(tnmc_env* env, cudaStream_t stream, void* work, si
     return TNMC_E_UNSUPPORTED;
   }
   if (d.z2) {
-    TNMC_CUDA_TRY(cudaFuncSetAttribute(build_env_z2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    build_env_z2_kernel<<<1, kBuildThreads, smem, stream>>>(a);
+    // One instance: the parity sectors on two SMs (a batch has an instance for every SM instead),
+    // unless the matrices are so small that the cluster barriers cost more.  One SM / two: 16 x 48,
+    // chi 32 451 / 366 ms; 10 x 20, chi 64 135 / 113; 12 x 12, chi 16 15.0 / 14.4; 8 x 8, chi 8
+    // 2.67 / 2.77.
+    const bool pair = d.P >= 16;
+    auto kern = pair ? build_env_z2_pair_kernel : build_env_z2_kernel;
+    TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<pair ? 2 : 1, kBuildThreads, smem, stream>>>(a);
   } else {
     TNMC_CUDA_TRY(cudaFuncSetAttribute(build_env_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     build_env_kernel<<<1, kBuildThreads, smem, stream>>>(a);
