@@ -1203,7 +1203,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=20.0)
     ap.add_argument("--cpu-batch", type=int, default=0)
-    ap.add_argument("--plain-batch", type=int, default=2 * 152 * 64)   # one full wave of the FP64 kernel
+    ap.add_argument("--plain-batch", type=int, default=2 * 152 * 64)   # 128 samples per SM
     ap.add_argument("--no-plain", action="store_true")
     ap.add_argument("--iters", type=int, default=30, help="iterations of the Delta trajectory (c3d)")
     ap.add_argument("--gauge", default=None, choices=["spin", "bond"],
