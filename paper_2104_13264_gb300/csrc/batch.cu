@@ -353,13 +353,17 @@ tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
     } else {
       const int SB = f32_block(rows, p->max_P, nsm);
       S = 8 * SB;
-      NW = f32_warps(p->max_P, max_Lx, SB, std::max(1, std::min(4, p->tile / S)), (size_t)max_optin - 1024);
-      if (NW == 0) {
-        tnmc_set_error("batched sampler needs %zu bytes of shared memory per CTA (device allows %d)",
-                       f32_smem(p->max_P, max_Lx, SB, 1).total, max_optin);
+      auto need = [&](int nw) {
+        return f32_smem_largest(p->n, [&](int i) { return p->envs[i]->d.P; },
+                                [&](int i) { return p->envs[i]->d.Lx; }, SB, nw);
+      };
+      NW = std::max(1, std::min(4, p->tile / S));
+      while (NW > 1 && need(NW) > (size_t)max_optin - 1024) NW >>= 1;
+      const size_t smem = need(NW);
+      if (smem > (size_t)max_optin - 1024) {
+        tnmc_set_error("batched sampler needs %zu bytes of shared memory per CTA (device allows %d)", smem, max_optin);
         return TNMC_E_UNSUPPORTED;
       }
-      const size_t smem = f32_smem(p->max_P, max_Lx, SB, NW).total;
       p->smem_of[q] = smem;
       st = by_f32_block(SB, p->max_P, [&](auto sb, auto xbm) -> tnmc_status {
         auto kern = sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value>;

@@ -660,6 +660,18 @@ inline int f32_warps(int P, int Lx, int SB, int want, size_t max_smem) {
   while (NW > 0 && f32_smem(P, Lx, SB, NW).total > max_smem) NW >>= 1;
   return NW;
 }
+// The same for a CTA that takes tiles of several lattices (P(i), Lx(i), i < n).  Each tile lays
+// the memory out for its own lattice, and the size does not grow with P alone (the ring holds three
+// tensors up to P = 32 and two above), so the reservation is the largest over the lattices.
+template <class FP, class FL>
+size_t f32_smem_largest(int n, FP&& P, FL&& Lx, int SB, int NW) {
+  size_t m = 0;
+  for (int i = 0; i < n; ++i) {
+    const size_t t = f32_smem(P(i), Lx(i), SB, NW).total;
+    if (t > m) m = t;
+  }
+  return m;
+}
 
 template <class F>
 tnmc_status by_f32_block(int SB, int P, F&& f) {
