@@ -627,7 +627,24 @@ __device__ bool jacobi_rows(double* J, int m, int n, int ld, double* d, int* fla
 
 // ---------------------------------------------------------------------------
 // 3. Right-to-left SVD sweep with truncation.
+//
+// Numbers that overflow (beta |J| in the hundreds) set the status and go on: the buffers are laid
+// out for the truncated bonds, so every bond is truncated whatever the values are.
 // ---------------------------------------------------------------------------
+// Norm of a row from its sum of squares.  NaN counts as zero, which keeps the ranks by norm a
+// permutation of the rows (a NaN compares false with everything).
+__device__ __forceinline__ double row_norm(double s, int32_t* status) {
+  if (s >= 0.0) return sqrt(s);
+  set_status(status, TNMC_E_NUMERIC);
+  return 0.0;
+}
+// The largest norm as the scale of a truncation; 1 where it is zero or infinite.
+__device__ __forceinline__ double usable_scale(double smax, int32_t* status) {
+  if (smax > 0.0 && isfinite(smax)) return smax;
+  if (threadIdx.x == 0) set_status(status, TNMC_E_NUMERIC);
+  return 1.0;
+}
+
 __device__ double svd_sweep(const BuildArgs& a, Shared& sh, int r) {
   const int Lx = a.Lx, P = a.P;
   const size_t slot_sz = (size_t)8 * P * P;
@@ -653,7 +670,7 @@ __device__ double svd_sweep(const BuildArgs& a, Shared& sh, int r) {
       double s = 0.0;
       for (int x = lane; x < n; x += 32) s += J[i * ld + x] * J[i * ld + x];
       s = warp_sum(s);
-      if (lane == 0) nrm[i] = sqrt(s);
+      if (lane == 0) nrm[i] = row_norm(s, a.status);
     }
     __syncthreads();
     // rank of each row by norm (descending; ties by index) -> sel[rank] = row
@@ -678,11 +695,7 @@ __device__ double svd_sweep(const BuildArgs& a, Shared& sh, int r) {
       if (rank >= kk) dsc += nrm[j] * nrm[j];
     }
     dsc = block_sum(dsc, sh.red);
-    const double smax = nrm[sh.sel[0]];
-    if (!(smax > 0.0) || !isfinite(smax)) {
-      if (threadIdx.x == 0) set_status(a.status, TNMC_E_NUMERIC);
-      return logs;
-    }
+    const double smax = usable_scale(nrm[sh.sel[0]], a.status);
     double* svr = a.sv + ((size_t)r * (Lx + 1) + c) * P;
     for (int j = threadIdx.x; j < P; j += blockDim.x) svr[j] = (j < kk) ? nrm[sh.sel[j]] / sqrt(tot) : 0.0;
     if (threadIdx.x == 0) a.disc[r * (Lx + 1) + c] = dsc / tot;
@@ -893,7 +906,7 @@ __device__ void var_split(const BuildArgs& a, Shared& sh, const VarWork& v, int 
     double s = 0.0;
     for (int x = lane; x < len; x += 32) s += J[i * ld + x] * J[i * ld + x];
     s = warp_sum(s);
-    if (lane == 0) nrm[i] = sqrt(s);
+    if (lane == 0) nrm[i] = row_norm(s, a.status);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < rows; i += blockDim.x) {
@@ -906,11 +919,7 @@ __device__ void var_split(const BuildArgs& a, Shared& sh, const VarWork& v, int 
     if (rank < kk) sh.sel[rank] = i;
   }
   __syncthreads();
-  const double smax = nrm[sh.sel[0]];
-  if (!(smax > 0.0) || !isfinite(smax)) {
-    if (threadIdx.x == 0) set_status(a.status, TNMC_E_NUMERIC);
-    return;
-  }
+  const double smax = usable_scale(nrm[sh.sel[0]], a.status);
   if (record) {
     double tot = 0.0, dsc = 0.0;
     for (int i = threadIdx.x; i < rows; i += blockDim.x) tot += nrm[i] * nrm[i];
@@ -1433,7 +1442,7 @@ __device__ double svd_sweep_z2(const BuildArgs& a, ShZ2& sh, int r) {
       double sq = 0.0;
       for (int x = lane; x < n; x += 32) sq += J[i * ld + x] * J[i * ld + x];
       sq = warp_sum(sq);
-      if (lane == 0) nrm[i] = sqrt(sq);
+      if (lane == 0) nrm[i] = row_norm(sq, a.status);
     }
     __syncthreads();
     // global rank (descending norm, ties by index); kept rows listed sector by sector
@@ -1466,11 +1475,7 @@ __device__ double svd_sweep_z2(const BuildArgs& a, ShZ2& sh, int r) {
     }
     tot = block_sum(tot, sh.red);
     dsc = block_sum(dsc, sh.red);
-    const double smax = nrm[sh.sel[0]];
-    if (!(smax > 0.0) || !isfinite(smax)) {
-      if (threadIdx.x == 0) set_status(a.status, TNMC_E_NUMERIC);
-      return logs;
-    }
+    const double smax = usable_scale(nrm[sh.sel[0]], a.status);
     double* svr = a.sv + ((size_t)r * (Lx + 1) + c) * P;
     for (int j = threadIdx.x; j < P; j += blockDim.x) svr[j] = (j < kk) ? nrm[sh.sel[j]] / sqrt(tot) : 0.0;
     if (threadIdx.x == 0) a.disc[r * (Lx + 1) + c] = dsc / tot;

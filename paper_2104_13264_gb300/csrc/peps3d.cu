@@ -137,9 +137,25 @@ __device__ bool orth_rows(VJ J, int m, int n, VJ d) {
   return converged;
 }
 
-// sel[0..k) = the k rows of largest norm (descending; ties by index).
+// A scale to divide by: 1 in the place of zero, infinity and NaN (returns false).  Compressions go
+// on with it, because the buffers are laid out for truncated bonds whatever the values are.
+template <typename T>
+__device__ __forceinline__ bool usable_scale3(T& s) {
+  if (s > 0 && isfinite((double)s)) return true;
+  s = T(1);
+  return false;
+}
+
+// sel[0..k) = the k <= m rows of largest norm (descending; ties by index).  A NaN norm becomes zero
+// (returns false): it compares false with everything, and the ranks have to be a permutation.
 template <typename T, typename VJ>
-__device__ void select_rows(VJ d, int m, int k, int* sel) {
+__device__ bool select_rows(VJ d, int m, int k, int* sel) {
+  bool ok = true;
+  for (int i = 0; i < m; ++i)
+    if (!(d[i] >= 0)) {
+      d[i] = T(0);
+      ok = false;
+    }
   for (int i = 0; i < m; ++i) {
     int rank = 0;
     const T di = d[i];
@@ -149,6 +165,7 @@ __device__ void select_rows(VJ d, int m, int k, int* sel) {
     }
     if (rank < k) sel[rank] = i;
   }
+  return ok;
 }
 
 // Successive SVD of an MPS of ns sites (site i at M.at(i * cap), layout [dl][p][dr]):
@@ -203,7 +220,7 @@ __device__ int mps_compress(V<T> M, int64_t cap, int ns, int* dl, const int* pp,
       const T aa = sm[e] < 0 ? -sm[e] : sm[e];
       sc = aa > sc ? aa : sc;
     }
-    if (!(sc > 0) || !isfinite((double)sc)) return TNMC_E_NUMERIC;
+    if (!usable_scale3(sc)) err = TNMC_E_NUMERIC;
     lg += log((double)sc);
     for (int q = 0; q < k; ++q)
       for (int x = 0; x < len; ++x) Mi[(int64_t)x * k + q] = J[(int64_t)q * len + x];
@@ -228,9 +245,9 @@ __device__ int mps_compress(V<T> M, int64_t cap, int ns, int* dl, const int* pp,
     if (!orth_rows<T>(J, a, len, d)) err = TNMC_E_NUMERIC;
     int k = a < len ? a : len;
     k = kmax < k ? kmax : k;
-    select_rows<T>(d, a, k, sel);
-    const T smax = d[sel[0]];
-    if (!(smax > 0) || !isfinite((double)smax)) return TNMC_E_NUMERIC;
+    if (!select_rows<T>(d, a, k, sel)) err = TNMC_E_NUMERIC;
+    T smax = d[sel[0]];
+    if (!usable_scale3(smax)) err = TNMC_E_NUMERIC;
     for (int j = 0; j < k; ++j) {
       const T nj = d[sel[j]];
       const T inv = nj > Tol3<T>::null * smax ? T(1) / nj : T(0);
@@ -320,7 +337,7 @@ __device__ int mps_compress_shared(V<T> M, int64_t cap, int ns, int* dl, const i
       const T aa = sm[e] < 0 ? -sm[e] : sm[e];
       sc = aa > sc ? aa : sc;
     }
-    if (!(sc > 0) || !isfinite((double)sc)) return TNMC_E_NUMERIC;
+    if (!usable_scale3(sc)) err = TNMC_E_NUMERIC;
     lg += log((double)sc);
     for (int q = 0; q < k; ++q)
       for (int x = 0; x < len; ++x) Mi[(int64_t)x * k + q] = J[q * len + x];
@@ -346,9 +363,9 @@ __device__ int mps_compress_shared(V<T> M, int64_t cap, int ns, int* dl, const i
     if (!orth_rows<T>(J, a, len, d)) err = TNMC_E_NUMERIC;
     int k = a < len ? a : len;
     k = kmax < k ? kmax : k;
-    select_rows<T>(d, a, k, sel);
-    const T smax = d[sel[0]];
-    if (!(smax > 0) || !isfinite((double)smax)) return TNMC_E_NUMERIC;
+    if (!select_rows<T>(d, a, k, sel)) err = TNMC_E_NUMERIC;
+    T smax = d[sel[0]];
+    if (!usable_scale3(smax)) err = TNMC_E_NUMERIC;
     for (int j = 0; j < k; ++j) {
       const T nj = d[sel[j]];
       const T inv = nj > Tol3<T>::null * smax ? T(1) / nj : T(0);
@@ -1141,7 +1158,7 @@ __device__ int mps_compress_w(T* M, int64_t cap, int ns, int* dl, const int* pp,
       sc = aa > sc ? aa : sc;
     }
     sc = wmax<G>(sc, gm);
-    if (!(sc > 0) || !isfinite((double)sc)) return TNMC_E_NUMERIC;
+    if (!usable_scale3(sc)) err = TNMC_E_NUMERIC;
     lg += log((double)sc);
     for (int e = lane; e < k * len; e += G) {
       const int x = e / k, q = e % k;
@@ -1171,17 +1188,10 @@ __device__ int mps_compress_w(T* M, int64_t cap, int ns, int* dl, const int* pp,
     if (!orth_rows_w<G>(J, a, len, d, lane, gm)) err = TNMC_E_NUMERIC;
     int k = a < len ? a : len;
     k = kmax < k ? kmax : k;
-    if (lane == 0) {
-      for (int r = 0; r < a; ++r) {
-        int rank = 0;
-        const T dr_ = d[r];
-        for (int j = 0; j < a; ++j) rank += (d[j] > dr_) || (d[j] == dr_ && j < r);
-        if (rank < k) sel[rank] = r;
-      }
-    }
+    if (lane == 0 && !select_rows<T>(d, a, k, sel)) err = TNMC_E_NUMERIC;
     __syncwarp(gm);
-    const T smax = d[sel[0]];
-    if (!(smax > 0) || !isfinite((double)smax)) return TNMC_E_NUMERIC;
+    T smax = d[sel[0]];
+    if (!usable_scale3(smax)) err = TNMC_E_NUMERIC;
     for (int e = lane; e < k * len; e += G) {
       const int j = e / len, y = e % len;
       const T nj = d[sel[j]];
