@@ -81,16 +81,34 @@ bool is_integer_array(const double* p, size_t n) {
   return true;
 }
 
-// Exponent of the fixed-point couplings: the largest magnitude times the number of terms of
-// H stays below 2^61 units.
+// Exponent of the fixed-point couplings: the smallest for which the sum of all magnitudes, rounded,
+// stays below 2^63 units (every partial sum of H then fits 64 bits).  Against the sum of 53-bit
+// couplings in FP64, mean error of random configurations: 128 x 128 Gaussian couplings 3.0e-13 ->
+// 1.4e-13, with one field of 1e3 2.5e-12 -> 1.9e-13, of 1e6 2.1e-9 -> 0; 256 x 256 5.5e-13 -> 8.3e-13.
 int fixed_point_exponent(const tnmc_lattice& lat, size_t nJh, size_t nJv, size_t nh) {
-  double mx = 0.0;
-  for (size_t i = 0; i < nJh; ++i) mx = fmax(mx, fabs(lat.Jh[i]));
-  for (size_t i = 0; i < nJv; ++i) mx = fmax(mx, fabs(lat.Jv[i]));
-  for (size_t i = 0; i < nh; ++i) mx = fmax(mx, fabs(lat.h[i]));
-  if (mx == 0.0) return 0;
-  const int terms = ilogb((double)(nJh + nJv + nh)) + 1;
-  return ilogb(mx) + 1 + terms - 61;
+  double sum = 0.0;
+  int e0 = 0;      // magnitudes are taken relative to 2^e0: their sum cannot overflow
+  for (int pass = 0; pass < 2; ++pass) {
+    double mx = 0.0;
+    auto add = [&](const double* p, size_t n) {
+      for (size_t i = 0; i < n; ++i) {
+        if (pass == 0) mx = fmax(mx, fabs(p[i]));
+        else sum += ldexp(fabs(p[i]), -e0);
+      }
+    };
+    add(lat.Jh, nJh);
+    add(lat.Jv, nJv);
+    add(lat.h, nh);
+    if (pass == 0) {
+      if (mx == 0.0) return 0;
+      e0 = ilogb(mx);
+    }
+  }
+  const double terms = (double)(nJh + nJv + nh);
+  int e = ilogb(sum) + 1;      // sum < 2^e
+  // roundings of the couplings (half a unit each) and of `sum` itself
+  if (ldexp(sum, 63 - e) * (1.0 + 1e-7) + terms >= 0x1p63) ++e;
+  return e0 + e - 63;
 }
 
 }  // namespace

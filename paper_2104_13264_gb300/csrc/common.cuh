@@ -46,7 +46,7 @@ struct DeviceEnv {
   const float* K32;
   const __nv_bfloat16* L16;
   const __nv_bfloat16* R16;
-  // couplings in 64-bit fixed point, J = q 2^qexp with |H| < 2^61 2^qexp: the energy of a
+  // couplings in 64-bit fixed point, J = q 2^qexp with sum |q| < 2^63: the energy of a
   // configuration is an exact integer sum (integer couplings stay exact)
   const int64_t* qJh;
   const int64_t* qJv;
