@@ -238,6 +238,8 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
     return TNMC_E_NOMEM;
   }
   d.qexp = fixed_point_exponent(*lat, nJh, nJv, nh);
+  d.strong = 0;
+  for (size_t i = 0; i < nJv; ++i) d.strong |= beta * fabs(lat->Jv[i]) > kStrongBond;
   auto put = [&](const double* src, size_t cnt, size_t o, size_t oq) {
     if (cnt == 0) return;
     memcpy(image.data() + o, src, cnt * 8);

@@ -69,7 +69,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 // cta_ns[2 i], cta_ns[2 i + 1]: when CTA i started and when it found no item left (global
 // timer, ns): the load balance of the launch is sum(busy) / (grid x makespan).
 // FP32: a CTA of NW warps takes an item at a time, NW 8 SB samples at once.
-template <int SB, int XBM>
+template <int SB, int XBM, bool EDGE>
 __global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM))
     sample_batched_f32_kernel(const SampleArgs<float>* __restrict__ tab, const int2* __restrict__ items, int64_t nitems,
                               int tile, unsigned long long* counter, float* scratch, size_t stack_elems,
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM))
     }
     __syncthreads();
     for (int64_t base = (int64_t)it.y * tile; base < (int64_t)(it.y + 1) * tile && base < a.B; base += step)
-      sample_f32_tile<SB, XBM>(a, base, smem_raw, stack);
+      sample_f32_tile<SB, XBM, EDGE>(a, base, smem_raw, stack);
   }
   if (threadIdx.x == 0) cta_ns[2 * blockIdx.x + 1] = global_ns();
 }
@@ -266,9 +266,11 @@ struct tnmc_batch {
   int grid = 0;
   size_t smem = 0, stack_elems = 0, scratch_bytes = 0, arena_bytes = 0;   // stack_elems: per sample
   int max_P = 1;
+  bool strong = false;     // a lattice has strong vertical bonds
   // samples per warp, warps per CTA and shared memory of the proposal [0] and chain [1] launches
   int s_warp[2] = {0, 0}, warps[2] = {1, 1};
   size_t smem_of[2] = {0, 0};
+  tnmc::F32Plan f32[2] = {};      // FP32: the two launches' kernels
   tnmc::Allocator alloc;   // the hook current when the plan was created
   // device memory: one arena for the tables, one for the per-CTA stacks
   void* arena = nullptr;
@@ -351,24 +353,25 @@ tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
         return TNMC_OK;
       });
     } else {
-      const int SB = f32_block(rows, p->max_P, nsm);
-      S = 8 * SB;
-      auto need = [&](int nw) {
-        return f32_smem_largest(p->n, [&](int i) { return p->envs[i]->d.P; },
-                                [&](int i) { return p->envs[i]->d.Lx; }, SB, nw);
-      };
-      NW = std::max(1, std::min(4, p->tile / S));
-      while (NW > 1 && need(NW) > (size_t)max_optin - 1024) NW >>= 1;
-      const size_t smem = need(NW);
-      if (smem > (size_t)max_optin - 1024) {
-        tnmc_set_error("batched sampler needs %zu bytes of shared memory per CTA (device allows %d)", smem, max_optin);
+      F32Plan& f = p->f32[q];
+      f = f32_plan(
+          rows, p->max_P, p->strong, nsm, (size_t)max_optin - 1024,
+          [&](int SB, int nw, bool edge) {
+            return f32_smem_largest(p->n, [&](int i) { return p->envs[i]->d.P; },
+                                    [&](int i) { return p->envs[i]->d.Lx; }, SB, nw, edge);
+          },
+          [&](int SB) { return std::max(1, std::min(4, p->tile / (8 * SB))); });
+      if (f.NW == 0) {
+        tnmc_set_error("batched sampler needs %zu bytes of shared memory per CTA (device allows %d)", f.smem, max_optin);
         return TNMC_E_UNSUPPORTED;
       }
-      p->smem_of[q] = smem;
-      st = by_f32_block(SB, p->max_P, [&](auto sb, auto xbm) -> tnmc_status {
-        auto kern = sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value>;
-        TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, smem));
+      S = 8 * f.SB;
+      NW = f.NW;
+      p->smem_of[q] = f.smem;
+      st = by_f32_block(f, p->max_P, [&](auto sb, auto xbm, auto edge) -> tnmc_status {
+        auto kern = sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value, decltype(edge)::value>;
+        TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
+        TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, f.smem));
         return TNMC_OK;
       });
     }
@@ -439,8 +442,8 @@ tnmc_status dispatch_batched(tnmc_batch* p, bool chains, const int8_t* spins_in,
   }
   const tnmc_status st = batched_begin<float>(p, chains, spins_in, spins_out, logq, energy, flags, s);
   if (st != TNMC_OK) return st;
-  return by_f32_block(S / 8, p->max_P, [&](auto sb, auto xbm) -> tnmc_status {
-    sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value><<<p->grid, threads, smem, s>>>(
+  return by_f32_block(p->f32[q], p->max_P, [&](auto sb, auto xbm, auto edge) -> tnmc_status {
+    sample_batched_f32_kernel<decltype(sb)::value, decltype(xbm)::value, decltype(edge)::value><<<p->grid, threads, smem, s>>>(
         static_cast<const SampleArgs<float>*>(tab), items, nitems, p->tile, p->d_counter + q,
         static_cast<float*>(p->scratch), p->stack_elems, p->d_cta_ns);
     TNMC_CUDA_TRY(cudaGetLastError());
@@ -523,6 +526,7 @@ tnmc_status tnmc_batch_create(int n, tnmc_env* const* envs, const int64_t* B, in
     p->items_prop += (B[i] + tile - 1) / tile;
     p->items_chain += (chains + tile - 1) / tile;
     p->max_P = std::max(p->max_P, d.P);
+    p->strong = p->strong || d.strong;
     max_Lx = std::max(max_Lx, d.Lx);
     max_stack = std::max(max_stack, precision == TNMC_F64 ? (size_t)(d.Lx + 1) * d.P : tnmc::f32_stack_floats(d.P, d.Lx));
     cost[i] = instance_cost(d);

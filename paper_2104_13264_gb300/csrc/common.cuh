@@ -11,6 +11,10 @@ namespace tnmc {
 
 constexpr int kMaxChi = 64;       // largest supported bond dimension
 constexpr int kMaxPad = 64;       // padded bond stride P <= 64
+// Vertical bonds beta |Jv| beyond this make the FP32 kernels rescale their vectors at once.  Otherwise
+// they divide a vector's exponent out one or two steps later and hold products of up to three
+// field factors exp(beta |Jv|), which reach the ends of FP32 (2^127) from 29 on.
+constexpr double kStrongBond = 20.0;
 
 // ---------------------------------------------------------------------------
 // Environment held on the device.
@@ -52,6 +56,7 @@ struct DeviceEnv {
   const int64_t* qJv;
   const int64_t* qh;
   int qexp;
+  int strong;            // beta max |Jv| > kStrongBond
   int32_t* status;       // device status word
 };
 
@@ -206,6 +211,11 @@ tnmc_status tnmc_launch_bond_sampling(tnmc_env* env, cudaStream_t stream);
 tnmc_status tnmc_launch_sample(const tnmc_env* env, int precision, int64_t B, uint64_t seed,
                                uint64_t sample_offset, const int8_t* spins_in, int8_t* spins_out,
                                double* logq, double* energy, int32_t* flags, cudaStream_t stream);
+// The FP64 and FP32 samplers with their stacks in `fixed_scratch` (null: in the env's scratch)
+tnmc_status tnmc_launch_sample_simt(const tnmc_env* env, int precision, int64_t B, uint64_t seed,
+                                    uint64_t sample_offset, const int8_t* spins_in, int8_t* spins_out,
+                                    double* logq, double* energy, int32_t* flags, void* fixed_scratch,
+                                    size_t fixed_bytes, cudaStream_t stream);
 tnmc_status tnmc_launch_derive_tc(tnmc_env* env, cudaStream_t stream);
 size_t tnmc_tc_tile_bytes();
 tnmc_status tnmc_launch_sample_tc(const tnmc_env* env, int64_t B, uint64_t seed, uint64_t offset,

@@ -25,6 +25,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "sample_args.cuh"
 #include "umma.cuh"
@@ -193,22 +195,23 @@ __device__ __forceinline__ void f32_contract(const float* M, int P, int dK, cons
 __device__ __forceinline__ void refresh(int& a, int& b, int& c) { asm volatile("" : "+r"(a), "+r"(b), "+r"(c)); }
 
 // Shared memory of a CTA of NW warps: the tensor ring (nbuf tiles and slack for the reads of
-// unused outputs), the field factors and bond dimensions of two rows, then per warp X [P][S],
-// the per-sample state of the finished rows, w [2][S], the scales [S] and two rows of spin masks.
+// unused outputs), the field factors and bond dimensions of two rows (EDGE: neither, they are read
+// from global memory), then per warp X [P][S], the per-sample state of the finished rows, w [2][S],
+// the scales [S] and two rows of spin masks.
 struct F32Smem {
   int nbuf;
   size_t ring, fer, bond, warp0, warp_bytes, total;
 };
-inline __host__ __device__ F32Smem f32_smem(int P, int Lx, int SB, int NW) {
+inline __host__ __device__ F32Smem f32_smem(int P, int Lx, int SB, int NW, bool edge) {
   F32Smem m;
   m.nbuf = P > 32 ? 2 : 3;
   const int S = 8 * SB, NO = (S + 31) / 32;
   m.ring = 0;
   size_t o = ((size_t)m.nbuf * P * 2 * P + 128) * sizeof(float);
   m.fer = o;
-  o += (size_t)4 * Lx * sizeof(float);
+  if (!edge) o += (size_t)4 * Lx * sizeof(float);
   m.bond = o;
-  o += (size_t)2 * (Lx + 1) * sizeof(int);
+  if (!edge) o += (size_t)2 * (Lx + 1) * sizeof(int);
   o = (o + 15) & ~(size_t)15;
   m.warp0 = o;
   m.warp_bytes = (((size_t)P * S + 3 * S) * sizeof(float) + (size_t)3 * 32 * NO * 8 +
@@ -231,7 +234,9 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // Samples base0 .. of one instance by the whole CTA (NW = blockDim.x / 32 warps, S each).
 // `stack`: the CTA's vector stacks, NW S f32_stack_floats(P, Lx) floats.
-template <int SB, int XBM>
+// EDGE: rows so wide that their field factors and bond dimensions in shared memory would cost the
+// SM warps, and strong vertical bonds.
+template <int SB, int XBM, bool EDGE>
 __device__ void sample_f32_tile(const SampleArgs<float>& a, int64_t base0, unsigned char* smem, float* stack) {
   using Ln = F32Lane<SB>;
   constexpr int S = Ln::S, NO = Ln::NO, LP = S >= 32 ? 1 : 32 / S;
@@ -239,7 +244,7 @@ __device__ void sample_f32_tile(const SampleArgs<float>& a, int64_t base0, unsig
   const int Lx = a.e.Lx, Ly = a.e.Ly, P = a.e.P;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x >> 5;
   const int lane_id = lane, lane_sg = lane & 7, lane_g = lane >> 3;
-  const F32Smem lay = f32_smem(P, Lx, SB, NW);
+  const F32Smem lay = f32_smem(P, Lx, SB, NW, EDGE);
   float* ring = reinterpret_cast<float*>(smem);
   float* fer2 = reinterpret_cast<float*>(smem + lay.fer);
   int* bond2 = reinterpret_cast<int*>(smem + lay.bond);
@@ -311,10 +316,16 @@ __device__ void sample_f32_tile(const SampleArgs<float>& a, int64_t base0, unsig
   };
 
   for (int r = 0; r < Ly; ++r) {
-    float* fer = fer2 + (size_t)(r & 1) * 2 * Lx;
-    int* bond = bond2 + (size_t)(r & 1) * (Lx + 1);
-    for (int c = threadIdx.x; c <= Lx; c += blockDim.x) bond[c] = a.e.bond[r * (Lx + 1) + c];
-    for (int c = threadIdx.x; c < 2 * Lx; c += blockDim.x) fer[c] = r == 0 ? 1.0f : a.fe[(size_t)r * Lx * 2 + c];
+    const float* fer = a.fe + (size_t)r * Lx * 2;      // 1 on row 0
+    const int* bond = a.e.bond + (size_t)r * (Lx + 1);
+    if constexpr (!EDGE) {
+      float* sfer = fer2 + (size_t)(r & 1) * 2 * Lx;
+      int* sbond = bond2 + (size_t)(r & 1) * (Lx + 1);
+      for (int c = threadIdx.x; c <= Lx; c += blockDim.x) sbond[c] = a.e.bond[r * (Lx + 1) + c];
+      for (int c = threadIdx.x; c < 2 * Lx; c += blockDim.x) sfer[c] = r == 0 ? 1.0f : a.fe[(size_t)r * Lx * 2 + c];
+      fer = sfer;
+      bond = sbond;
+    }
     const bool snake = a.e.order == 1 && (r & 1);
     if (a.spins_in && alive) {
       for (int c = lane; c < Lx; c += 32) {
@@ -380,6 +391,24 @@ __device__ void sample_f32_tile(const SampleArgs<float>& a, int64_t base0, unsig
           elag[b] = exponent_f32(__float_as_int(mb[b]));
         }
       });
+      if (EDGE && a.e.strong) {      // f 2^-elag, or f times the vector, may leave FP32: rescale it now
+        const int XB = f32_xb(dX);
+#pragma unroll 1
+        for (int x = 0; x < XB; ++x) {
+          float v[SB];
+#pragma unroll
+          for (int q = 0; q < SB; q += Ln::VS) {
+            float* o = out + ((x * SB + q) / Ln::VS * 32 + lane_id) * Ln::VS;
+            load_run<Ln::VS>(o, &v[q]);
+#pragma unroll
+            for (int b = q; b < q + Ln::VS; ++b) v[b] *= pow2_f32(-elag[b]);
+            store_run<Ln::VS>(o, &v[q]);
+          }
+          if (XB * lane_g + x < dX) Ln::store(X + (XB * lane_g + x) * S, lane_sg, v);
+        }
+#pragma unroll
+        for (int b = 0; b < SB; ++b) elag[b] = 0;
+      }
       __syncwarp();
     }
     // ---- second sweep: the draws ----
@@ -632,13 +661,13 @@ __device__ void sample_f32_tile(const SampleArgs<float>& a, int64_t base0, unsig
 // 8-sample block at 168 registers took 7.99 instead of 4.95 ms).
 __host__ __device__ constexpr int f32_min_ctas(int SB, int XBM) { return SB * XBM >= 32 ? 2 : 3; }
 
-template <int SB, int XBM>
+template <int SB, int XBM, bool EDGE>
 __global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM)) sample_f32_kernel(SampleArgs<float> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t step = (int64_t)(blockDim.x >> 5) * (8 * SB);
   float* stack = a.scratch + (size_t)blockIdx.x * step * f32_stack_floats(a.e.P, a.e.Lx);
   for (int64_t base = blockIdx.x * step; base < a.B; base += gridDim.x * step)
-    sample_f32_tile<SB, XBM>(a, base, smem_raw, stack);
+    sample_f32_tile<SB, XBM, EDGE>(a, base, smem_raw, stack);
 }
 
 // Samples per lane for `total` samples on `nsm` SMs at pad P.  Large blocks need fewer
@@ -654,32 +683,54 @@ inline int f32_block(int64_t total, int P, int nsm) {
   while (SB > 1 && (total + 8 * SB - 1) / (8 * SB) < 3 * (int64_t)nsm) SB >>= 1;
   return SB;
 }
-// Warps per CTA whose shared memory fits (0: not even one).
-inline int f32_warps(int P, int Lx, int SB, int want, size_t max_smem) {
-  int NW = want;
-  while (NW > 0 && f32_smem(P, Lx, SB, NW).total > max_smem) NW >>= 1;
-  return NW;
+// Bonds per output lane that the kernel of block SB is compiled for.
+__host__ __device__ constexpr int f32_xbm(int SB, int P) { return SB == 8 ? 4 : SB == 4 ? (P <= 16 ? 4 : 8) : P <= 32 ? 8 : 16; }
+
+// The launch of `total` samples: samples per lane, warps per CTA (0: not even one fits), the kernel's
+// form and its shared memory.  need(SB, NW, edge): bytes of a CTA; want(SB): most warps per CTA.
+struct F32Plan {
+  int SB, NW;
+  bool edge;
+  size_t smem;
+};
+template <class Need, class Want>
+F32Plan f32_plan(int64_t total, int P, bool strong, int nsm, size_t max_smem, Need&& need, Want&& want) {
+  F32Plan p{f32_block(total, P, nsm), 0, strong, 0};
+  if (strong && p.SB == 8) p.SB = 4;
+  for (p.NW = want(p.SB); p.NW > 0; p.NW >>= 1) {
+    p.smem = need(p.SB, p.NW, p.edge);
+    if (p.smem <= max_smem) break;
+  }
+  return p;
 }
-// The same for a CTA that takes tiles of several lattices (P(i), Lx(i), i < n).  Each tile lays
-// the memory out for its own lattice, and the size does not grow with P alone (the ring holds three
+
+// Shared memory of a CTA that takes tiles of several lattices (P(i), Lx(i), i < n).  Each tile lays it
+// out for its own lattice, and the size does not grow with P alone (the ring holds three
 // tensors up to P = 32 and two above), so the reservation is the largest over the lattices.
 template <class FP, class FL>
-size_t f32_smem_largest(int n, FP&& P, FL&& Lx, int SB, int NW) {
+size_t f32_smem_largest(int n, FP&& P, FL&& Lx, int SB, int NW, bool edge) {
   size_t m = 0;
   for (int i = 0; i < n; ++i) {
-    const size_t t = f32_smem(P(i), Lx(i), SB, NW).total;
+    const size_t t = f32_smem(P(i), Lx(i), SB, NW, edge).total;
     if (t > m) m = t;
   }
   return m;
 }
 
+// f(IntF<SB>, IntF<XBM>, bool constant EDGE) for a plan's kernel (EDGE: at most 4 samples per lane)
 template <class F>
-tnmc_status by_f32_block(int SB, int P, F&& f) {
-  switch (SB) {
-    case 8: return f(IntF<8>{}, IntF<4>{});
-    case 4: return P <= 16 ? f(IntF<4>{}, IntF<4>{}) : f(IntF<4>{}, IntF<8>{});
-    case 2: return P <= 32 ? f(IntF<2>{}, IntF<8>{}) : f(IntF<2>{}, IntF<16>{});
-    default: return P <= 32 ? f(IntF<1>{}, IntF<8>{}) : f(IntF<1>{}, IntF<16>{});
+tnmc_status by_f32_block(const F32Plan& p, int P, F&& f) {
+  auto form = [&](auto sb, auto xbm) -> tnmc_status {
+    constexpr int kSB = decltype(sb)::value;
+    if constexpr (kSB < 8)
+      if (p.edge) return f(sb, xbm, std::true_type{});
+    return f(sb, xbm, std::false_type{});
+  };
+  switch (p.SB) {
+    case 8: return form(IntF<8>{}, IntF<4>{});
+    case 4: return P <= 16 ? form(IntF<4>{}, IntF<4>{}) : form(IntF<4>{}, IntF<8>{});
+    case 2: return P <= 32 ? form(IntF<2>{}, IntF<8>{}) : form(IntF<2>{}, IntF<16>{});
+    default: return P <= 32 ? form(IntF<1>{}, IntF<8>{}) : form(IntF<1>{}, IntF<16>{});
   }
 }
 

@@ -58,53 +58,66 @@ __global__ void fields_kernel(DeviceEnv e, double* fe, float* fe32) {
   }
 }
 
+// Scratch of a launch: the caller's fixed bytes, or the env's, grown as needed.
+struct SimtScratch {
+  const tnmc_env* env;
+  void* fixed;
+  size_t bytes;
+};
+
+// The largest grid of at most `grid` CTAs whose stacks (per_cta bytes each) the scratch holds.
+tnmc_status take_scratch(const SimtScratch& s, int64_t& grid, size_t per_cta, cudaStream_t stream, void** out) {
+  if (s.fixed) {
+    const int64_t fit = (int64_t)(s.bytes / per_cta);
+    if (grid > fit) grid = fit;
+    *out = s.fixed;
+    return TNMC_OK;
+  }
+  tnmc_env* me = const_cast<tnmc_env*>(s.env);
+  const tnmc_status st = grow_scratch(me, (size_t)grid * per_cta, stream, "sampler");
+  *out = me->scratch.ptr;
+  return st;
+}
+
 // FP64: one warp per CTA, S samples per warp (f64_tile_samples).
 template <int LS, int SB>
-tnmc_status launch_sample_f64(const tnmc_env* env, SampleArgs<double> a, int nsm, cudaStream_t stream) {
+tnmc_status launch_sample_f64(const SimtScratch& scr, SampleArgs<double> a, int nsm, cudaStream_t stream) {
   constexpr int S = LS * SB;
-  const DeviceEnv& d = env->d;
   auto kern = sample_f64_kernel<LS, SB>;
-  const size_t smem = f64_tile_smem(d.P, d.Lx, S);
+  const size_t smem = f64_tile_smem(a.e.P, a.e.Lx, S);
   if (smem > 48 * 1024) TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem));
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (a.B + S - 1) / S;
   if (grid > (int64_t)nsm * per_sm) grid = (int64_t)nsm * per_sm;
-  tnmc_env* me = const_cast<tnmc_env*>(env);
-  const tnmc_status gs = grow_scratch(me, (size_t)grid * (d.Lx + 1) * d.P * S * sizeof(double), stream, "sampler");
-  if (gs != TNMC_OK) return gs;
-  a.scratch = static_cast<double*>(me->scratch.ptr);
+  void* scratch = nullptr;
+  const tnmc_status st = take_scratch(scr, grid, (size_t)(a.e.Lx + 1) * a.e.P * S * sizeof(double), stream, &scratch);
+  if (st != TNMC_OK) return st;
+  a.scratch = static_cast<double*>(scratch);
   kern<<<(unsigned)grid, 32, smem, stream>>>(a);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }
 
-// FP32: CTAs of up to 4 warps, 8 SB samples per warp (f32_block).
-template <int SB, int XBM>
-tnmc_status launch_sample_f32(const tnmc_env* env, SampleArgs<float> a, int nsm, int max_smem, cudaStream_t stream) {
-  const DeviceEnv& d = env->d;
-  auto kern = sample_f32_kernel<SB, XBM>;
-  const int NW = f32_warps(d.P, d.Lx, SB, 4, (size_t)max_smem);
-  if (NW == 0) {
-    tnmc_set_error("sampler needs %zu bytes of shared memory per CTA (device allows %d)",
-                   f32_smem(d.P, d.Lx, SB, 1).total, max_smem);
-    return TNMC_E_UNSUPPORTED;
-  }
-  const size_t smem = f32_smem(d.P, d.Lx, SB, NW).total;
-  TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+// FP32: CTAs of up to 4 warps, 8 SB samples per warp (f32_plan).
+template <int SB, int XBM, bool EDGE>
+tnmc_status launch_sample_f32(const SimtScratch& scr, SampleArgs<float> a, const F32Plan& p, int nsm,
+                              cudaStream_t stream) {
+  auto kern = sample_f32_kernel<SB, XBM, EDGE>;
+  TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
   int per_sm = 0;
-  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, smem));
+  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * p.NW, p.smem));
   if (per_sm < 1) per_sm = 1;
-  const int64_t tile = (int64_t)NW * 8 * SB;
+  const int64_t tile = (int64_t)p.NW * 8 * SB;
   int64_t grid = (a.B + tile - 1) / tile;
   if (grid > (int64_t)nsm * per_sm) grid = (int64_t)nsm * per_sm;
-  tnmc_env* me = const_cast<tnmc_env*>(env);
-  const tnmc_status gs =
-      grow_scratch(me, (size_t)grid * tile * f32_stack_floats(d.P, d.Lx) * sizeof(float), stream, "sampler");
-  if (gs != TNMC_OK) return gs;
-  a.scratch = static_cast<float*>(me->scratch.ptr);
-  kern<<<(unsigned)grid, 32 * NW, smem, stream>>>(a);
+  void* scratch = nullptr;
+  const tnmc_status st =
+      take_scratch(scr, grid, (size_t)tile * f32_stack_floats(a.e.P, a.e.Lx) * sizeof(float), stream, &scratch);
+  if (st != TNMC_OK) return st;
+  a.scratch = static_cast<float*>(scratch);
+  kern<<<(unsigned)grid, 32 * p.NW, p.smem, stream>>>(a);
   TNMC_CUDA_TRY(cudaGetLastError());
   return TNMC_OK;
 }
@@ -154,12 +167,13 @@ tnmc_status tnmc_launch_rederive_f32(tnmc_env* env, cudaStream_t stream) {
   return TNMC_OK;
 }
 
-tnmc_status tnmc_launch_sample(const tnmc_env* env, int precision, int64_t B, uint64_t seed,
-                               uint64_t offset, const int8_t* spins_in, int8_t* spins_out, double* logq,
-                               double* energy, int32_t* flags, cudaStream_t stream) {
+tnmc_status tnmc_launch_sample_simt(const tnmc_env* env, int precision, int64_t B, uint64_t seed, uint64_t offset,
+                                    const int8_t* spins_in, int8_t* spins_out, double* logq, double* energy,
+                                    int32_t* flags, void* fixed_scratch, size_t fixed_bytes, cudaStream_t stream) {
   using namespace tnmc;
   const DeviceEnv& d = env->d;
   if (B == 0) return TNMC_OK;
+  const SimtScratch scr{env, fixed_scratch, fixed_bytes};
   int dev = 0, nsm = 0, max_smem = 0;
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -167,19 +181,39 @@ tnmc_status tnmc_launch_sample(const tnmc_env* env, int precision, int64_t B, ui
   if (precision == TNMC_F64) {
     const SampleArgs<double> a{d, d.M64, d.R64, d.fe, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
     switch (f64_tile_samples(B, d.P, nsm)) {
-      case 32: return launch_sample_f64<8, 4>(env, a, nsm, stream);
-      case 16: return launch_sample_f64<8, 2>(env, a, nsm, stream);
-      case 8: return launch_sample_f64<8, 1>(env, a, nsm, stream);
-      case 4: return launch_sample_f64<4, 1>(env, a, nsm, stream);
-      default: return launch_sample_f64<2, 1>(env, a, nsm, stream);
+      case 32: return launch_sample_f64<8, 4>(scr, a, nsm, stream);
+      case 16: return launch_sample_f64<8, 2>(scr, a, nsm, stream);
+      case 8: return launch_sample_f64<8, 1>(scr, a, nsm, stream);
+      case 4: return launch_sample_f64<4, 1>(scr, a, nsm, stream);
+      default: return launch_sample_f64<2, 1>(scr, a, nsm, stream);
     }
   }
-  if (precision == TNMC_F32) {
-    const SampleArgs<float> a{d, d.K32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
-    return by_f32_block(f32_block(B, d.P, nsm), d.P, [&](auto sb, auto xbm) -> tnmc_status {
-      return launch_sample_f32<decltype(sb)::value, decltype(xbm)::value>(env, a, nsm, max_smem, stream);
-    });
+  const SampleArgs<float> a{d, d.K32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
+  const size_t stack = f32_stack_floats(d.P, d.Lx) * sizeof(float);
+  const F32Plan p = f32_plan(
+      B, d.P, d.strong, nsm, (size_t)max_smem,
+      [&](int SB, int NW, bool edge) { return f32_smem(d.P, d.Lx, SB, NW, edge).total; },
+      [&](int SB) {      // a CTA's stacks have to fit a fixed scratch
+        int NW = 4;
+        while (fixed_scratch && NW > 1 && (size_t)NW * 8 * SB * stack > fixed_bytes) NW >>= 1;
+        return NW;
+      });
+  if (p.NW == 0) {
+    tnmc_set_error("sampler needs %zu bytes of shared memory per CTA (device allows %d)", p.smem, max_smem);
+    return TNMC_E_UNSUPPORTED;
   }
+  return by_f32_block(p, d.P, [&](auto sb, auto xbm, auto edge) -> tnmc_status {
+    return launch_sample_f32<decltype(sb)::value, decltype(xbm)::value, decltype(edge)::value>(scr, a, p, nsm, stream);
+  });
+}
+
+tnmc_status tnmc_launch_sample(const tnmc_env* env, int precision, int64_t B, uint64_t seed, uint64_t offset,
+                               const int8_t* spins_in, int8_t* spins_out, double* logq, double* energy,
+                               int32_t* flags, cudaStream_t stream) {
+  if (B == 0) return TNMC_OK;
+  if (precision == TNMC_F64 || precision == TNMC_F32)
+    return tnmc_launch_sample_simt(env, precision, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr,
+                                   0, stream);
   if (precision == TNMC_BF16)
     return tnmc_launch_sample_tc(env, B, seed, offset, spins_in, spins_out, logq, energy, flags, stream);
   tnmc_set_error("unknown precision %d", precision);

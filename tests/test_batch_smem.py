@@ -23,14 +23,15 @@ int main() {
   const int pads[] = {4, 8, 16, 20, 28, 32, 36, 40, 48, 64}, widths[] = {1, 8, 31, 32, 33, 64, 250, 1024};
   const int np = 10, nl = 8;
   long bad = 0, shrinks = 0, cases = 0;
+  for (int edge = 0; edge < 2; ++edge)
   for (int SB = 1; SB <= 8; SB *= 2)
     for (int NW = 1; NW <= 4; NW *= 2)
       for (int i = 0; i < np * nl; ++i)
         for (int j = 0; j < np * nl; ++j, ++cases) {
           const int P[2] = {pads[i / nl], pads[j / nl]}, L[2] = {widths[i % nl], widths[j % nl]};
-          const size_t r = f32_smem_largest(2, [&](int k) { return P[k]; }, [&](int k) { return L[k]; }, SB, NW);
-          for (int k = 0; k < 2; ++k) bad += f32_smem(P[k], L[k], SB, NW).total > r;
-          const size_t corner = f32_smem(P[0] > P[1] ? P[0] : P[1], L[0] > L[1] ? L[0] : L[1], SB, NW).total;
+          const size_t r = f32_smem_largest(2, [&](int k) { return P[k]; }, [&](int k) { return L[k]; }, SB, NW, edge);
+          for (int k = 0; k < 2; ++k) bad += f32_smem(P[k], L[k], SB, NW, edge).total > r;
+          const size_t corner = f32_smem(P[0] > P[1] ? P[0] : P[1], L[0] > L[1] ? L[0] : L[1], SB, NW, edge).total;
           shrinks += r > corner;
         }
   printf("%ld %ld %ld\n", cases, bad, shrinks);
@@ -49,7 +50,7 @@ def test_reservation_covers_every_lattice(tmp_path):
                     "--expt-relaxed-constexpr", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
     cases, bad, shrinks = map(int, out.split())
-    assert cases == 4 * 3 * 80 * 80
+    assert cases == 2 * 4 * 3 * 80 * 80
     assert bad == 0
     # the pairs for which the layout of the largest pad and width would have been too small exist
     assert shrinks > 0

@@ -1,0 +1,43 @@
+"""Strong vertical bonds (needs a GB300): beta |Jv| up to the end of FP32's range.
+
+A row's field factors are exp(+-beta Jv).  The FP32 sampler stays unflagged as long as a single
+factor fits FP32 (beta |Jv| < 88), and its log q agrees with FP64 to 1e-4 relative (the precision's
+stated bound), whatever the signs of neighbouring bonds are; a batch equals the single calls.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _lattice(Ly, Lx, beta, seed):
+    """Vertical bonds of magnitude 0.9 to 1, everything else of order 1 / beta."""
+    r = np.random.default_rng(seed)
+    Jh = 0.7 / beta * r.standard_normal((Ly, Lx - 1))
+    Jv = r.choice([-1.0, 1.0], size=(Ly - 1, Lx)) * r.uniform(0.9, 1.0, size=(Ly - 1, Lx))
+    h = 0.3 / beta * r.standard_normal((Ly, Lx))
+    return Jh, Jv, h
+
+
+@pytest.mark.parametrize("beta", [19.0, 21.0, 30.0, 48.0, 84.0])
+@pytest.mark.parametrize("Ly,Lx,chi", [(6, 9, 4), (7, 13, 20), (7, 14, 40)])
+def test_f32_strong_bonds(Ly, Lx, chi, beta):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2104_13264_gb300 import binding as B
+    env = B.Env(*_lattice(Ly, Lx, beta, chi), beta, chi, precisions=("f64", "f32"))
+    for n in (300, 20000):
+        for order in ("raster", "snake"):
+            env.set_order(order)
+            sp, lq, E, fl = B.sample(env, n, seed=5, precision="f32")
+            lq64, _, fl64 = B.logq(env, sp, precision="f64")
+            assert not fl.any() and not fl64.any()
+            np.testing.assert_allclose(lq.cpu().numpy(), lq64.cpu().numpy(), rtol=1e-4)
+        plan = B.Batch([env, env], [n, n], chains=n // 2, precision="f32")
+        plan.set_step(5, 0)
+        out = plan.sample(plan.alloc_proposals())
+        assert torch.equal(plan.view(out[0], 0), sp) and torch.equal(plan.rows(out[1], 0), lq)
+        plan.free()
+    env.free()
