@@ -18,8 +18,8 @@
 // lanes (lane quadrant w % 4) at different columns, 16 columns per load -- and writes the next
 // A operand straight back to TMEM.  Warp 8 issues the UMMAs; warp 9 refills the ring of
 // environment tiles and makes the sites' Philox words one left step ahead.  The two epilogue
-// halves exchange their partial maxima (every other right step) or partial dot products
-// (left steps) through shared memory and take identical decisions from identical sums.
+// halves exchange their partial maxima (every other right step; every one with strong
+// vertical bonds) or partial dot products (left steps) through shared memory and take identical decisions from identical sums.
 // Every rescaling is by a power of two, which leaves the arithmetic of q unchanged: right
 // vectors by their max, left vectors by the drawn weight w(s).
 //
@@ -118,10 +118,10 @@ __device__ inline void pair_sync(int warp) {
   asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory");
 }
 
-// STAGED: the row's field factors and the masks of its own spins in shared memory.  Otherwise
-// the factors are read from the environment and the masks kept behind the stacks in global
-// scratch.
-template <bool STAGED>
+// The row's field factors and the masks of its own spins are in shared memory.  EDGE: wide rows,
+// where the factors are read from the environment and the masks kept behind the stacks in global
+// scratch, and strong vertical bonds.
+template <bool EDGE>
 __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -133,12 +133,12 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
   // environment tiles whose copy was issued
   int64_t* cnt = reinterpret_cast<int64_t*>(misc + 4);
   float* xw = reinterpret_cast<float*>(misc + 6);   // left steps: [2 halves][2][128] partial w(-), w(+)
-  float* xmb = xw + 4 * kTile;                      // right steps: [2 halves][128] partial max
+  float* xmb = xw + 4 * kTile;                      // right steps: [step parity][2 halves][128] partial max
   const int Lx = a.e.Lx, Ly = a.e.Ly;
   uint32_t* xs = reinterpret_cast<uint32_t*>(xw + 8 * kTile);   // [2 pairs][2 sites][2][128]: 64-bit uniforms
   uint32_t* prev = xs + 8 * kTile;                              // [Lx][4]: spins of the row above, one bit a sample
-  uint32_t* cur = STAGED ? prev + 4 * Lx
-                         : reinterpret_cast<uint32_t*>(a.stack + (size_t)gridDim.x * Lx * (2 * 8 * kTile)) +
+  uint32_t* cur = !EDGE ? prev + 4 * Lx
+                        : reinterpret_cast<uint32_t*>(a.stack + (size_t)gridDim.x * Lx * (2 * 8 * kTile)) +
                                (size_t)blockIdx.x * 4 * Lx;
 
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
     };
     for (int r = 0; r < Ly && !abort; ++r) {
       const float* fe_row = a.fe + (size_t)r * Lx * 2;     // [Lx][2]: field factors of the row; 1 on row 0
-      if constexpr (STAGED) {
+      if constexpr (!EDGE) {
         float* sfe = reinterpret_cast<float*>(cur + 4 * Lx);
         for (int q = tid; q < 2 * Lx; q += kThreads) sfe[q] = fe_row[q];
         fe_row = sfe;
@@ -349,11 +349,15 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
           // above): the UMMA formed both u halves, the epilogue selects one ----
           // every other step rescales by the power of two of the previous A operand's largest entry
           // (the odd steps record both halves' partial maxima, exchanged through the step barrier):
-          // the operand stays within two steps' growth of [1, 2)
-          const bool record = i & 1;
+          // the operand stays within two steps' growth of [1, 2) and the accumulator within three,
+          // which fit FP32 up to beta |Jv| = 29.  With stronger bonds (EDGE) every step records and
+          // rescales: the accumulator holds two steps' growth, up to 44.
+          const bool every = EDGE && a.e.strong;
+          const bool record = every || (i & 1), scale = every || !(i & 1);
+          const int rd = every ? ((i + 1) & 1) * (2 * kTile) : 0;      // the previous step's maxima
           float2 sc = make_float2(1.0f, 1.0f);
-          if (!record && i > 0) {
-            const float mprev = fmaxf(xmb[t], xmb[kTile + t]);
+          if (scale && i > 0) {
+            const float mprev = fmaxf(xmb[rd + t], xmb[rd + kTile + t]);
             if (mprev > 0x1.0p-126f && mprev < INFINITY) sc.x = sc.y = pow2f(-ilogb_f(mprev));
           }
           float m4[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // four independent chains (max is exact)
@@ -370,6 +374,10 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
               v[q] = make_float2(__uint_as_float(up ? e[2 * q] : d[2 * q]), __uint_as_float(up ? e[2 * q + 1] : d[2 * q + 1]));
+            if (EDGE && every) {
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[q] = umma::f2_mul(v[q], sc);
+            }
             if (record) {
 #pragma unroll
               for (int q = 0; q < 8; ++q) m4[q & 3] = fmaxf(m4[q & 3], fmaxf(fabsf(v[q].x), fabsf(v[q].y)));
@@ -384,7 +392,8 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
           }
           if (c == 1) store_unit(a_hi, a_lo, h);           // the left sweep starts from Lambda_0 = e_0
           umma::tmem_wait_st();
-          if (record) xmb[h * kTile + t] = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+          if (record)
+            xmb[(every ? (i & 1) * (2 * kTile) : 0) + h * kTile + t] = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
         } else {
           // ---- left-sweep epilogue: w(s) = f(s) <U[s], R_{c+1}>, draw, Lambda_{c+1} ----
           cp_async_wait_all();
@@ -612,14 +621,14 @@ tnmc_status tnmc_launch_sample_tc(const tnmc_env* env, int64_t B, uint64_t seed,
   // 509 columns).  Measured, chi 16, 6 rows, 65536 samples, staged / not: 96 columns 4.59 / 4.68 ms,
   // 256 columns 18.2 (one CTA) / 12.5 (two), 600 columns 42.9 / 44.5.
   const size_t row_bytes = (size_t)6 * d.Lx * sizeof(uint32_t);
-  const bool staged = smem + row_bytes <= (size_t)max_optin &&
+  const bool staged = !d.strong && smem + row_bytes <= (size_t)max_optin &&
                       (2 * (smem + row_bytes + 1024) <= (size_t)smem_sm || 2 * (smem + 1024) > (size_t)smem_sm);
   if (staged) smem += row_bytes;
   if (smem > (size_t)max_optin) {
     tnmc_set_error("tensor-core sampler needs %zu bytes of shared memory (device allows %d)", smem, max_optin);
     return TNMC_E_UNSUPPORTED;
   }
-  auto kern = staged ? sample_tc_kernel<true> : sample_tc_kernel<false>;
+  auto kern = staged ? sample_tc_kernel<false> : sample_tc_kernel<true>;
   TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)cudaSharedmemCarveoutMaxShared));

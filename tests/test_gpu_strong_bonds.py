@@ -2,7 +2,8 @@
 
 A row's field factors are exp(+-beta Jv).  The FP32 sampler stays unflagged as long as a single
 factor fits FP32 (beta |Jv| < 88), and its log q agrees with FP64 to 1e-4 relative (the precision's
-stated bound), whatever the signs of neighbouring bonds are; a batch equals the single calls.
+stated bound), whatever the signs of neighbouring bonds are; a batch equals the single calls.  The
+BF16 sampler, whose accumulator holds two factors, does the same up to 44.
 """
 import numpy as np
 import pytest
@@ -40,4 +41,18 @@ def test_f32_strong_bonds(Ly, Lx, chi, beta):
         out = plan.sample(plan.alloc_proposals())
         assert torch.equal(plan.view(out[0], 0), sp) and torch.equal(plan.rows(out[1], 0), lq)
         plan.free()
+    env.free()
+
+
+@pytest.mark.parametrize("beta", [19.0, 21.0, 32.0, 42.0])
+@pytest.mark.parametrize("Ly,Lx,chi", [(6, 9, 4), (7, 13, 20), (7, 14, 40)])
+def test_bf16_strong_bonds(Ly, Lx, chi, beta):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2104_13264_gb300 import binding as B
+    env = B.Env(*_lattice(Ly, Lx, beta, chi), beta, chi, precisions=("f64", "bf16"))
+    sp, lq, E, fl = B.sample(env, 300, seed=5, precision="bf16")
+    lq64, _, fl64 = B.logq(env, sp, precision="f64")
+    assert not fl.any() and not fl64.any()
+    np.testing.assert_allclose(lq.cpu().numpy(), lq64.cpu().numpy(), rtol=1e-4)
     env.free()
