@@ -219,16 +219,16 @@ __device__ __forceinline__ void site_gradient(const float* V, const float* W, co
   }
 }
 
-// STAGED: the row's field factors and bond dimensions in shared memory; rows too wide for that
-// (P = 64: more than 2630 columns) read them from global memory.
-template <bool STAGED>
+// The row's field factors and bond dimensions are in shared memory.  EDGE: rows too wide for that
+// (P = 64: more than 2630 columns), which read them from global memory, and strong vertical bonds.
+template <bool EDGE>
 __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const unsigned kFull = 0xffffffffu;
   const int Lx = a.e.Lx, Ly = a.e.Ly, P = a.e.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sl = lane & 7, ol = (lane >> 3) + 4 * warp;      // samples 4 sl .. 4 sl + 3, outputs XB ol ..
-  const GradSmem lay = grad_smem(P, Lx, STAGED);
+  const GradSmem lay = grad_smem(P, Lx, !EDGE);
   float* ring = reinterpret_cast<float*>(smem_raw);
   float* set0 = reinterpret_cast<float*>(smem_raw + lay.set);
   const size_t set_sz = (size_t)6 * P * kGStride;
@@ -301,6 +301,34 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
       }
       if (lane < 8) store_run<4>(mpart + (par * 4 + warp) * kGT + 4 * sl, m);
     };
+    // Strong vertical bonds: a vector just written (rows x of X and of the stack slot St, this
+    // thread's samples) is rescaled at once, by the exponent of its own largest entry (e on return).
+    // The weights then hold one field factor instead of up to three (f_c, and those of Lambda_c
+    // and R_{c+1}), whose product leaves FP32 from beta |Jv| = 29 on.
+    auto rescale_now = [&](int par, int dX, float* X, float* St, int (&e)[4]) {
+      __syncthreads();
+      lag(par, e);
+      by_outputs(dX, [&](auto xbc) {
+        constexpr int XB = decltype(xbc)::value;
+        for (int x = XB * ol; x < XB * ol + XB && x < dX; ++x) {
+          float v[4];
+          load4(X + x * kGStride + 4 * sl, v);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) v[b] *= pow2_f32(-e[b]);
+          store_run<4>(X + x * kGStride + 4 * sl, v);
+          store_run<4>(St + x * kGT + 4 * sl, v);
+        }
+      });
+    };
+    // the exponent of the vector a step reads: lag, or 0 where rescale_now has divided it out
+    auto lag_of = [&](int par, int (&e)[4]) {
+      if (EDGE && a.e.strong) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) e[b] = 0;
+      } else {
+        lag(par, e);
+      }
+    };
     auto put_one = [&](float* X) {       // the boundary vector: one row of ones
       if (tid < kGT) X[tid] = 1.0f;
       if (tid < 4 * kGT) mpart[tid] = 1.0f;      // parity 0
@@ -310,7 +338,7 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
       __syncthreads();
       const int* bond = a.e.bond + (size_t)r * (Lx + 1);
       const float* fer = a.fe + (size_t)r * Lx * 2;       // 1 on row 0
-      if constexpr (STAGED) {
+      if constexpr (!EDGE) {
         int* sbond = reinterpret_cast<int*>(smem_raw + lay.bond);
         float* sfer = reinterpret_cast<float*>(smem_raw + lay.fer);
         for (int c = tid; c <= Lx; c += kGThreads) sbond[c] = bond[c];
@@ -346,7 +374,7 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
           float acc[2][XB][4], m[4];
           int e[4];
           contract_out<XB>(M, P, dK, X, ol, sl, acc);
-          lag(step & 1, e);
+          lag_of(step & 1, e);
 #pragma unroll
           for (int b = 0; b < 4; ++b) {
             const bool u = (up >> (4 * sl + b)) & 1u;
@@ -370,6 +398,11 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
           if (ol == 0) *reinterpret_cast<int4*>(ekp + c * kGT + 4 * sl) = make_int4(-e[0], -e[1], -e[2], -e[3]);
           put_max((step + 1) & 1, m);
         });
+        if (EDGE && a.e.strong) {
+          int e[4];
+          rescale_now((step + 1) & 1, dX, Xn, Rs + c * slot, e);
+          if (ol == 0) *reinterpret_cast<int4*>(ekp + c * kGT + 4 * sl) = make_int4(-e[0], -e[1], -e[2], -e[3]);
+        }
       }
       // ---- 2. left sweep (forced) ----
       __syncthreads();
@@ -403,7 +436,7 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
           float acc[2][XB][4], m[4], w0[4], w1[4];
           int e[4];
           contract_out<XB>(M, P, dK, X, ol, sl, acc);
-          lag(step & 1, e);
+          lag_of(step & 1, e);
 #pragma unroll
           for (int b = 0; b < 4; ++b) {
             const bool u = (up >> (4 * sl + b)) & 1u, s = (sp >> (4 * sl + b)) & 1u;
@@ -441,6 +474,11 @@ __global__ void __launch_bounds__(kGThreads, 2) logq_grad_kernel(GradArgs a) {
             store_run<4>(wpart + (c & 1) * 8 * kGT + (2 * warp + 1) * kGT + 4 * sl, w1);
           }
         });
+        if (EDGE && a.e.strong) {
+          int e[4];
+          rescale_now((step + 1) & 1, dX, Xn, Ls + (c + 1) * slot, e);
+          if (ol == 0) *reinterpret_cast<int4*>(ek + c * kGT + 4 * sl) = make_int4(-e[0], -e[1], -e[2], -e[3]);
+        }
       }
       __syncthreads();
       finish_weights(Lx - 1);
@@ -654,13 +692,13 @@ tnmc_status tnmc_launch_logq_grad(const tnmc_env* env, int64_t B, const int8_t* 
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const bool staged = grad_smem(d.P, d.Lx, true).total <= (size_t)max_optin;
+  const bool staged = !d.strong && grad_smem(d.P, d.Lx, true).total <= (size_t)max_optin;
   const size_t smem = grad_smem(d.P, d.Lx, staged).total;
   if (smem > (size_t)max_optin) {
     tnmc_set_error("gradient kernel needs %zu bytes of shared memory (device allows %d)", smem, max_optin);
     return TNMC_E_UNSUPPORTED;
   }
-  auto kern = staged ? logq_grad_kernel<true> : logq_grad_kernel<false>;
+  auto kern = staged ? logq_grad_kernel<false> : logq_grad_kernel<true>;
   TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGThreads, smem));

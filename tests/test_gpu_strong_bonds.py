@@ -3,10 +3,13 @@
 A row's field factors are exp(+-beta Jv).  The FP32 sampler stays unflagged as long as a single
 factor fits FP32 (beta |Jv| < 88), and its log q agrees with FP64 to 1e-4 relative (the precision's
 stated bound), whatever the signs of neighbouring bonds are; a batch equals the single calls.  The
-BF16 sampler, whose accumulator holds two factors, does the same up to 44.
+BF16 sampler, whose accumulator holds two factors, does the same up to 44.  The gradient agrees with
+the oracle's on the same tensors to 1e-3 per site (the bound of the gradient parity tests).
 """
 import numpy as np
 import pytest
+
+from oracle import tnmc
 
 pytestmark = pytest.mark.gpu
 
@@ -55,4 +58,31 @@ def test_bf16_strong_bonds(Ly, Lx, chi, beta):
     lq64, _, fl64 = B.logq(env, sp, precision="f64")
     assert not fl.any() and not fl64.any()
     np.testing.assert_allclose(lq.cpu().numpy(), lq64.cpu().numpy(), rtol=1e-4)
+    env.free()
+
+
+@pytest.mark.parametrize("beta", [19.0, 21.0, 32.0, 42.0])
+@pytest.mark.parametrize("Ly,Lx,chi", [(6, 9, 4), (7, 13, 20), (7, 14, 40)])
+def test_grad_strong_bonds(Ly, Lx, chi, beta):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2104_13264_gb300 import binding as B
+    Jh, Jv, h = _lattice(Ly, Lx, beta, chi)
+    env = B.Env(Jh, Jv, h, beta, chi, precisions=("f64", "f32"))
+    P = env.info()["pad"]
+    ex = env.export()
+    bd = ex["bond_dims"]
+    ref = tnmc.Env(Lx, Ly, beta, chi, Jh, Jv, h)
+    ref.M = [[ex["tensors"][r, c, :bd[r, c], :, :bd[r, c + 1]].astype(np.float32).astype(np.float64)
+              for c in range(Lx)] for r in range(Ly)]
+    sp = B.sample(env, 40, seed=7)[0].cpu().numpy()
+    w = np.random.default_rng(chi).random(40)
+    _, G = tnmc.logq_grad(ref, sp, w)
+    grad = B.logq_backward(env, torch.from_numpy(sp).cuda(), torch.from_numpy(w).float().cuda())
+    g = grad.cpu().numpy().reshape(Ly, Lx, P, 2, P)
+    gmax = max(np.linalg.norm(G[r][c]) for r in range(Ly) for c in range(Lx))
+    for r in range(Ly):
+        for c in range(Lx):
+            got = g[r, c, :G[r][c].shape[0], :, :G[r][c].shape[2]]
+            assert np.linalg.norm(got - G[r][c]) <= 1e-3 * max(np.linalg.norm(G[r][c]), 1e-4 * gmax), (r, c)
     env.free()
