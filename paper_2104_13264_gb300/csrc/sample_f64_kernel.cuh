@@ -9,8 +9,8 @@
 //     of a contraction instruction carries a useful product even when a batch has few samples,
 //     and tiles of down to 2 samples give an SM the warps that fill its FP64 pipe.
 //   - Scalar work (normalisation, draw) runs on one lane per sample; log q is a running
-//     product with an integer exponent (one log per sample), the reciprocal is two Newton steps
-//     on rcp.approx, clamps, maxima, draws and power-of-two scales are integer operations, and
+//     product with an integer exponent (one log per sample), the division is two Newton steps
+//     on rcp.approx and a residual step, clamps, maxima, draws and power-of-two scales are integer operations, and
 //     the energy is an exact 64-bit fixed-point sum.
 // Measured against one thread per sample (64 per CTA): 23 x 29, chi = 13, 5000 samples 26.2 ->
 // 5.9 ms (73 % of the FP64 pipe); 64 lattices 32 x 32, chi = 16 with 32 samples each 47.9 -> 6.0 ms.
@@ -79,6 +79,13 @@ __device__ __forceinline__ double reciprocal_f64(double t) {
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(t));
   r = fma(r, fma(-t, r, 1.0), r);
   return fma(r, fma(-t, r, 1.0), r);
+}
+
+// w / t from r = reciprocal_f64(t): the product and one residual step (Markstein's correction), which
+// rounds to the nearest double; the product alone is off by up to two units in the last place.
+__device__ __forceinline__ double quotient_f64(double w, double t, double r) {
+  const double q = w * r;
+  return fma(fma(-q, t, w), r, q);
 }
 
 // +1 iff x < floor(p 2^64) (draw_plus), from the bits of p
@@ -295,21 +302,24 @@ __device__ void sample_f64_tile(const SampleArgs<double>& a, int64_t base, unsig
         const double tot = w0 + w1;
         const int te = (__double2hiint(tot) >> 20) & 0x7ff;
         const bool bad = te == 2047 || __double_as_longlong(tot) == 0;
-        double pplus = 0.5, pminus = 0.5;
-        if (!bad) {
-          if (te > 64 && te < 1980) {
-            const double ri = reciprocal_f64(tot);
-            pplus = w1 * ri;
-            pminus = w0 * ri;
-          } else {
-            pplus = w1 / tot;
-            pminus = w0 / tot;
-          }
-          if (__double_as_longlong(w0) == 0) pplus = 1.0;     // one weight zero: exact
-          if (__double_as_longlong(w1) == 0) pminus = 1.0;
+        // p(+) for the draw, p(s) for log q.  The draw compares with 64 uniform bits, which a unit in
+        // p's last place moves with probability 2^-53: the product will do, off the residual step's
+        // latency
+        const bool mid = te > 64 && te < 1980;
+        double ri = 0.0, pplus, pd;
+        if (mid) {
+          ri = reciprocal_f64(tot);
+          pplus = w1 * ri;
+        } else {
+          pplus = w1 / tot;
         }
+        if (__double_as_longlong(w0) == 0) pplus = 1.0;     // one weight zero: exact
+        if (bad) pplus = 0.5;
         const bool plus = a.spins_in ? (cur[c] >> so) & 1u : draw_plus_bits(pplus, word);
-        prod *= plus ? pplus : pminus;
+        const double wd = plus ? w1 : w0;
+        if (mid) pd = quotient_f64(wd, tot, ri);
+        else pd = bad ? 0.5 : wd / tot;
+        prod *= pd;
         {
           int hi = __double2hiint(prod);
           if ((hi >> 20) == 0 && prod != 0.0) {      // subnormal: exact shift into the normal range
