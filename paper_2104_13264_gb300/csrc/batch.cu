@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM))
 
 // FP64: one warp per CTA.  A work item of `tile` samples is handed out in tile / S warp tiles
 // (consecutive counter values), so that a batch of few samples still spreads over every SM.
-template <int LS, int SB>
+template <int LS, int SB, bool EDGE>
 __global__ void __launch_bounds__(32, kF64MinWarps) sample_batched_f64_kernel(const SampleArgs<double>* __restrict__ tab,
                                                                 const int2* __restrict__ items, int64_t nitems,
                                                                 int tile, unsigned long long* counter,
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(32, kF64MinWarps) sample_batched_f64_kernel(co
     const int2 it = items[k / per];
     const SampleArgs<double> a = tab[it.x];
     const int64_t base = (int64_t)it.y * tile + (int64_t)(k % per) * S;
-    if (base < a.B) sample_f64_tile<LS, SB>(a, base, smem_raw, stack);
+    if (base < a.B) sample_f64_tile<LS, SB, EDGE>(a, base, smem_raw, stack);
   }
   if (threadIdx.x == 0) cta_ns[2 * blockIdx.x + 1] = global_ns();
 }
@@ -270,7 +270,8 @@ struct tnmc_batch {
   // samples per warp, warps per CTA and shared memory of the proposal [0] and chain [1] launches
   int s_warp[2] = {0, 0}, warps[2] = {1, 1};
   size_t smem_of[2] = {0, 0};
-  tnmc::F32Plan f32[2] = {};      // FP32: the two launches' kernels
+  tnmc::F64Plan f64[2] = {};      // the two launches' kernels
+  tnmc::F32Plan f32[2] = {};
   tnmc::Allocator alloc;   // the hook current when the plan was created
   // device memory: one arena for the tables, one for the per-CTA stacks
   void* arena = nullptr;
@@ -315,25 +316,14 @@ const double* env_fe<double>(const tnmc_env* e) { return e->d.fe; }
 template <>
 const float* env_fe<float>(const tnmc_env* e) { return e->d.fe32; }
 
-template <class F>
-tnmc_status by_f64_tile(int S, F&& f) {
-  using tnmc::IntC;
-  switch (S) {
-    case 32: return f(IntC<8>{}, IntC<4>{});
-    case 16: return f(IntC<8>{}, IntC<2>{});
-    case 8: return f(IntC<8>{}, IntC<1>{});
-    case 4: return f(IntC<4>{}, IntC<1>{});
-    default: return f(IntC<2>{}, IntC<1>{});
-  }
-}
-
 // The tile shapes of the proposal and the chain launches, and a grid for both.
 tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
   using namespace tnmc;
-  int dev = 0, nsm = 0, max_optin = 0;
+  int dev = 0, nsm = 0, max_optin = 0, smem_sm = 0;
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
   const bool f64 = p->precision == TNMC_F64;
   int64_t grid = 1;
   size_t samples = 0;      // largest CTA tile
@@ -343,13 +333,14 @@ tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
     int S, NW = 1, per_sm = 0;
     tnmc_status st;
     if (f64) {
-      S = f64_tile_samples(rows, p->max_P, nsm);
-      const size_t smem = f64_tile_smem(p->max_P, max_Lx, S);
-      p->smem_of[q] = smem;
-      st = by_f64_tile(S, [&](auto ls, auto sb) -> tnmc_status {
-        auto kern = sample_batched_f64_kernel<decltype(ls)::value, decltype(sb)::value>;
-        if (smem > 48 * 1024) TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem));
+      F64Plan& f = p->f64[q];
+      f = f64_plan(rows, p->max_P, nsm, (size_t)smem_sm, [&](int s, bool edge) { return f64_tile_smem(p->max_P, max_Lx, s, edge); });
+      S = f.S;
+      p->smem_of[q] = f.smem;
+      st = by_f64_tile(f, [&](auto ls, auto sb, auto edge) -> tnmc_status {
+        auto kern = sample_batched_f64_kernel<decltype(ls)::value, decltype(sb)::value, decltype(edge)::value>;
+        if (f.smem > 48 * 1024) TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
+        TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, f.smem));
         return TNMC_OK;
       });
     } else {
@@ -432,8 +423,8 @@ tnmc_status dispatch_batched(tnmc_batch* p, bool chains, const int8_t* spins_in,
   if (p->precision == TNMC_F64) {
     const tnmc_status st = batched_begin<double>(p, chains, spins_in, spins_out, logq, energy, flags, s);
     if (st != TNMC_OK) return st;
-    return by_f64_tile(S, [&](auto ls, auto sb) -> tnmc_status {
-      sample_batched_f64_kernel<decltype(ls)::value, decltype(sb)::value><<<p->grid, threads, smem, s>>>(
+    return by_f64_tile(p->f64[q], [&](auto ls, auto sb, auto edge) -> tnmc_status {
+      sample_batched_f64_kernel<decltype(ls)::value, decltype(sb)::value, decltype(edge)::value><<<p->grid, threads, smem, s>>>(
           static_cast<const SampleArgs<double>*>(tab), items, nitems, p->tile, p->d_counter + q,
           static_cast<double*>(p->scratch), p->stack_elems, p->d_cta_ns);
       TNMC_CUDA_TRY(cudaGetLastError());

@@ -216,6 +216,10 @@ tnmc_status tnmc_launch_sample_simt(const tnmc_env* env, int precision, int64_t 
                                     uint64_t sample_offset, const int8_t* spins_in, int8_t* spins_out,
                                     double* logq, double* energy, int32_t* flags, void* fixed_scratch,
                                     size_t fixed_bytes, cudaStream_t stream);
+tnmc_status tnmc_launch_sample_f64(const tnmc_env* env, int64_t B, uint64_t seed, uint64_t sample_offset,
+                                   const int8_t* spins_in, int8_t* spins_out, double* logq, double* energy,
+                                   int32_t* flags, void* fixed_scratch, size_t fixed_bytes, int nsm, int smem_sm,
+                                   cudaStream_t stream);
 tnmc_status tnmc_launch_derive_tc(tnmc_env* env, cudaStream_t stream);
 size_t tnmc_tc_tile_bytes();
 tnmc_status tnmc_launch_sample_tc(const tnmc_env* env, int64_t B, uint64_t seed, uint64_t offset,

@@ -22,6 +22,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "sample_args.cuh"
 
@@ -139,9 +141,14 @@ __device__ __forceinline__ void f64_contract(const double* __restrict__ M, int P
 }
 
 // Shared memory of one warp tile: X [P][S] and U [2][P][S] doubles, the row's field factors [Lx][2], two rows
-// of spin masks [Lx] and the row's bond dimensions [Lx + 1].
-inline __host__ __device__ size_t f64_tile_smem(int P, int Lx, int S) {
-  return (3 * (size_t)P * S + 2 * (size_t)Lx) * sizeof(double) + ((size_t)3 * Lx + 1) * sizeof(uint32_t);
+// of spin masks [Lx] and the row's bond dimensions [Lx + 1].  EDGE: the factors and dimensions stay in
+// global memory, and a mask has only the bits of S samples.
+template <int S, bool EDGE>
+using F64Mask = std::conditional_t<!EDGE || (S > 16), uint32_t, std::conditional_t<(S > 8), uint16_t, uint8_t>>;
+inline __host__ __device__ size_t f64_tile_smem(int P, int Lx, int S, bool edge) {
+  const size_t work = 3 * (size_t)P * S * sizeof(double);
+  if (edge) return work + (size_t)2 * Lx * (S > 16 ? 4 : S > 8 ? 2 : 1);
+  return work + 2 * (size_t)Lx * sizeof(double) + ((size_t)3 * Lx + 1) * sizeof(uint32_t);
 }
 
 // The first dK rows of a site tensor into L1 (the warp's next contraction; its first loads
@@ -156,8 +163,10 @@ __device__ __forceinline__ void f64_prefetch(const double* M, int P, int dK, int
 
 // Samples base .. base+S-1 of the call (S = LS * SB <= 32, by one warp).  Bit s of a spin mask
 // is sample base + s; lane s < S keeps the scalar state of sample s.  `stack`: [Lx+1][P][S].
-template <int LS, int SB>
+// EDGE: wide rows (f64_tile_smem).
+template <int LS, int SB, bool EDGE>
 __device__ void sample_f64_tile(const SampleArgs<double>& a, int64_t base, unsigned char* smem, double* stack) {
+  using Mask = F64Mask<LS * SB, EDGE>;
   constexpr int LO = 32 / LS, S = LS * SB, MAXNX = 64 / LO / SB, LP = 32 / S;
   const unsigned kFull = 0xffffffffu;
   const int Lx = a.e.Lx, Ly = a.e.Ly, P = a.e.P;
@@ -165,10 +174,10 @@ __device__ void sample_f64_tile(const SampleArgs<double>& a, int64_t base, unsig
   const int so = lane % S;                      // the sample whose scalars this lane computes
   double* X = reinterpret_cast<double*>(smem);
   double* U = X + (size_t)P * S;
-  double* fer = U + 2 * (size_t)P * S;
-  uint32_t* prev = reinterpret_cast<uint32_t*>(fer + 2 * (size_t)Lx);
-  uint32_t* cur = prev + Lx;
-  int* bond = reinterpret_cast<int*>(cur + Lx);
+  double* sfer = U + 2 * (size_t)P * S;
+  Mask* prev = reinterpret_cast<Mask*>(sfer + (EDGE ? 0 : 2 * (size_t)Lx));
+  Mask* cur = prev + Lx;
+  int* sbond = reinterpret_cast<int*>(cur + Lx);
   const size_t n = (size_t)Lx * Ly, slot = (size_t)P * S;
   const uint64_t sample = a.offset + (uint64_t)(base + so);
   const int rows = (a.B - base) < S ? (int)(a.B - base) : S;
@@ -179,8 +188,14 @@ __device__ void sample_f64_tile(const SampleArgs<double>& a, int64_t base, unsig
   __syncwarp();
 
   for (int r = 0; r < Ly; ++r) {
-    for (int c = lane; c <= Lx; c += 32) bond[c] = a.e.bond[r * (Lx + 1) + c];
-    for (int c = lane; c < 2 * Lx; c += 32) fer[c] = r == 0 ? 1.0 : a.fe[(size_t)r * Lx * 2 + c];
+    const double* fer = a.fe + (size_t)r * Lx * 2;      // 1 on row 0
+    const int* bond = a.e.bond + (size_t)r * (Lx + 1);
+    if constexpr (!EDGE) {
+      for (int c = lane; c <= Lx; c += 32) sbond[c] = a.e.bond[r * (Lx + 1) + c];
+      for (int c = lane; c < 2 * Lx; c += 32) sfer[c] = r == 0 ? 1.0 : a.fe[(size_t)r * Lx * 2 + c];
+      fer = sfer;
+      bond = sbond;
+    }
     const size_t tstride = (size_t)P * 2 * P;
     const double* Lrow = a.L + (size_t)r * Lx * tstride;
     const double* Rrow = a.Rt + (size_t)r * Lx * tstride;
@@ -421,13 +436,13 @@ constexpr int kF64MinWarps = 12;
 
 // One warp per CTA: tiles are handed out in single warps, so that a few thousand samples
 // spread evenly over the SMs.  Scratch: one stack [Lx+1][P][S] per CTA.
-template <int LS, int SB>
+template <int LS, int SB, bool EDGE>
 __global__ void __launch_bounds__(32, kF64MinWarps) sample_f64_kernel(SampleArgs<double> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int S = LS * SB;
   double* stack = a.scratch + (size_t)blockIdx.x * (a.e.Lx + 1) * a.e.P * S;
   for (int64_t base = (int64_t)blockIdx.x * S; base < a.B; base += (int64_t)gridDim.x * S)
-    sample_f64_tile<LS, SB>(a, base, smem_raw, stack);
+    sample_f64_tile<LS, SB, EDGE>(a, base, smem_raw, stack);
 }
 
 // The tile shape (samples per warp) for `total` samples on `nsm` SMs at pad P.  Larger tiles
@@ -441,6 +456,43 @@ inline int f64_tile_samples(int64_t total, int P, int nsm) {
   int S = 32;
   while (S > 2 && (S / 8 * P > 64 || (total + S - 1) / S < (int64_t)kF64WarpsPerSM * nsm)) S >>= 1;
   return S;
+}
+
+// The launch of `total` samples: samples per warp, the kernel's form and its shared memory.
+// need(S, edge): bytes of a CTA of one warp.
+//
+// The EDGE form where the plain one would leave an SM fewer than its 12 warps (from about 500 columns
+// on: it costs up to 4 % itself), and there at most 16 samples where more would leave fewer than 7.
+// Measured, ms, plain form / the rule's: 8192 samples of 5 x 4096, chi 16 1190 / 212, of 4 x 2048, chi 8
+// 114 / 43; 32768 of 4 x 4096, chi 8 1130 / 282 (32 samples per warp: 350).
+struct F64Plan {
+  int S;
+  bool edge;
+  size_t smem;
+};
+template <class Need>
+F64Plan f64_plan(int64_t total, int P, int nsm, size_t smem_sm, Need&& need) {
+  F64Plan p{f64_tile_samples(total, P, nsm), false, 0};
+  auto warps = [&](int S, bool edge) { return (int)(smem_sm / (need(S, edge) + 1024)); };
+  p.edge = warps(p.S, false) < kF64MinWarps;
+  if (p.edge && p.S == 32 && warps(32, true) < 7) p.S = 16;
+  p.smem = need(p.S, p.edge);
+  return p;
+}
+
+// f(IntC<LS>, IntC<SB>, bool constant EDGE) for a plan's kernel
+template <class F>
+tnmc_status by_f64_tile(const F64Plan& p, F&& f) {
+  auto form = [&](auto ls, auto sb) -> tnmc_status {
+    return p.edge ? f(ls, sb, std::true_type{}) : f(ls, sb, std::false_type{});
+  };
+  switch (p.S) {
+    case 32: return form(IntC<8>{}, IntC<4>{});
+    case 16: return form(IntC<8>{}, IntC<2>{});
+    case 8: return form(IntC<8>{}, IntC<1>{});
+    case 4: return form(IntC<4>{}, IntC<1>{});
+    default: return form(IntC<2>{}, IntC<1>{});
+  }
 }
 
 }  // namespace

@@ -13,13 +13,12 @@
 //                 Lambda_{c+1} = f_c(s) U[s], rescaled by a power of two.
 // f_c(s) = exp(beta Jv[r-1][c] s_{r-1,c} s) carries the (exactly contracted)
 // product state of the rows above.  On the odd rows of the snake order the two sweeps
-// change roles (draws from the right).  The kernels are in sample_f64_kernel.cuh and
-// sample_f32_kernel.cuh.
+// change roles (draws from the right).  The kernels are in sample_f64_kernel.cuh (launched from
+// sample_f64.cu) and sample_f32_kernel.cuh.
 #include <math.h>
 
 #include "common.cuh"
 #include "sample_f32_kernel.cuh"
-#include "sample_f64_kernel.cuh"
 
 namespace tnmc {
 namespace {
@@ -56,48 +55,6 @@ __global__ void fields_kernel(DeviceEnv e, double* fe, float* fe32) {
     fe32[2 * i] = (float)d;
     fe32[2 * i + 1] = (float)s;
   }
-}
-
-// Scratch of a launch: the caller's fixed bytes, or the env's, grown as needed.
-struct SimtScratch {
-  const tnmc_env* env;
-  void* fixed;
-  size_t bytes;
-};
-
-// The largest grid of at most `grid` CTAs whose stacks (per_cta bytes each) the scratch holds.
-tnmc_status take_scratch(const SimtScratch& s, int64_t& grid, size_t per_cta, cudaStream_t stream, void** out) {
-  if (s.fixed) {
-    const int64_t fit = (int64_t)(s.bytes / per_cta);
-    if (grid > fit) grid = fit;
-    *out = s.fixed;
-    return TNMC_OK;
-  }
-  tnmc_env* me = const_cast<tnmc_env*>(s.env);
-  const tnmc_status st = grow_scratch(me, (size_t)grid * per_cta, stream, "sampler");
-  *out = me->scratch.ptr;
-  return st;
-}
-
-// FP64: one warp per CTA, S samples per warp (f64_tile_samples).
-template <int LS, int SB>
-tnmc_status launch_sample_f64(const SimtScratch& scr, SampleArgs<double> a, int nsm, cudaStream_t stream) {
-  constexpr int S = LS * SB;
-  auto kern = sample_f64_kernel<LS, SB>;
-  const size_t smem = f64_tile_smem(a.e.P, a.e.Lx, S);
-  if (smem > 48 * 1024) TNMC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = 0;
-  TNMC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, smem));
-  if (per_sm < 1) per_sm = 1;
-  int64_t grid = (a.B + S - 1) / S;
-  if (grid > (int64_t)nsm * per_sm) grid = (int64_t)nsm * per_sm;
-  void* scratch = nullptr;
-  const tnmc_status st = take_scratch(scr, grid, (size_t)(a.e.Lx + 1) * a.e.P * S * sizeof(double), stream, &scratch);
-  if (st != TNMC_OK) return st;
-  a.scratch = static_cast<double*>(scratch);
-  kern<<<(unsigned)grid, 32, smem, stream>>>(a);
-  TNMC_CUDA_TRY(cudaGetLastError());
-  return TNMC_OK;
 }
 
 // FP32: CTAs of up to 4 warps, 8 SB samples per warp (f32_plan).
@@ -174,20 +131,14 @@ tnmc_status tnmc_launch_sample_simt(const tnmc_env* env, int precision, int64_t 
   const DeviceEnv& d = env->d;
   if (B == 0) return TNMC_OK;
   const SimtScratch scr{env, fixed_scratch, fixed_bytes};
-  int dev = 0, nsm = 0, max_smem = 0;
+  int dev = 0, nsm = 0, max_smem = 0, smem_sm = 0;
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (precision == TNMC_F64) {
-    const SampleArgs<double> a{d, d.M64, d.R64, d.fe, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
-    switch (f64_tile_samples(B, d.P, nsm)) {
-      case 32: return launch_sample_f64<8, 4>(scr, a, nsm, stream);
-      case 16: return launch_sample_f64<8, 2>(scr, a, nsm, stream);
-      case 8: return launch_sample_f64<8, 1>(scr, a, nsm, stream);
-      case 4: return launch_sample_f64<4, 1>(scr, a, nsm, stream);
-      default: return launch_sample_f64<2, 1>(scr, a, nsm, stream);
-    }
-  }
+  TNMC_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+  if (precision == TNMC_F64)
+    return tnmc_launch_sample_f64(env, B, seed, offset, spins_in, spins_out, logq, energy, flags, fixed_scratch,
+                                  fixed_bytes, nsm, smem_sm, stream);
   const SampleArgs<float> a{d, d.K32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
   const size_t stack = f32_stack_floats(d.P, d.Lx) * sizeof(float);
   const F32Plan p = f32_plan(
