@@ -346,7 +346,7 @@ tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
     } else {
       F32Plan& f = p->f32[q];
       f = f32_plan(
-          rows, p->max_P, p->strong, nsm, (size_t)max_optin - 1024,
+          rows, p->max_P, p->strong, nsm, (size_t)max_optin - 1024, (size_t)smem_sm,
           [&](int SB, int nw, bool edge) {
             return f32_smem_largest(p->n, [&](int i) { return p->envs[i]->d.P; },
                                     [&](int i) { return p->envs[i]->d.Lx; }, SB, nw, edge);

@@ -202,6 +202,8 @@ struct F32Smem {
   int nbuf;
   size_t ring, fer, bond, warp0, warp_bytes, total;
 };
+template <int S, bool EDGE>
+using F32Mask = std::conditional_t<!EDGE || (S > 16), uint32_t, std::conditional_t<(S > 8), uint16_t, uint8_t>>;
 inline __host__ __device__ F32Smem f32_smem(int P, int Lx, int SB, int NW, bool edge) {
   F32Smem m;
   m.nbuf = P > 32 ? 2 : 3;
@@ -215,7 +217,7 @@ inline __host__ __device__ F32Smem f32_smem(int P, int Lx, int SB, int NW, bool 
   o = (o + 15) & ~(size_t)15;
   m.warp0 = o;
   m.warp_bytes = (((size_t)P * S + 3 * S) * sizeof(float) + (size_t)3 * 32 * NO * 8 +
-                  (size_t)2 * Lx * NO * sizeof(uint32_t) + 15) & ~(size_t)15;
+                  (size_t)2 * Lx * NO * (edge && S <= 16 ? S / 8 : 4) + 15) & ~(size_t)15;
   m.total = o + NW * m.warp_bytes;
   return m;
 }
@@ -254,8 +256,9 @@ __device__ void sample_f32_tile(const SampleArgs<float>& a, int64_t base0, unsig
   int64_t* st_e = st_qexp + 32 * NO;                                   // fixed-point energy
   float* wbuf = reinterpret_cast<float*>(st_e + 32 * NO);              // [2][S]
   float* mbuf = wbuf + 2 * S;              // [S]
-  uint32_t* prev = reinterpret_cast<uint32_t*>(mbuf + S);   // [Lx][NO]
-  uint32_t* cur = prev + (size_t)Lx * NO;
+  using Mask = F32Mask<S, EDGE>;
+  Mask* prev = reinterpret_cast<Mask*>(mbuf + S);   // [Lx][NO]
+  Mask* cur = prev + (size_t)Lx * NO;
   const size_t n = (size_t)Lx * Ly, tstride = (size_t)P * 2 * P;
   const size_t slot = (size_t)4 * f32_xb(P) * S;            // floats of one stack slot of a warp
   float* stk = stack + (size_t)warp * (Lx + 1) * slot;
@@ -688,20 +691,49 @@ __host__ __device__ constexpr int f32_xbm(int SB, int P) { return SB == 8 ? 4 : 
 
 // The launch of `total` samples: samples per lane, warps per CTA (0: not even one fits), the kernel's
 // form and its shared memory.  need(SB, NW, edge): bytes of a CTA; want(SB): most warps per CTA.
+//
+// f32_block's choice in the plain form, unless shared memory keeps fewer CTAs on an SM than the
+// registers allow (from about 1000 columns on): then, over both forms and all smaller blocks, the
+// least waves x time of a wave, where a wave of 8 / 4 / 2 / 1 samples per lane takes 1.45 / 1.15 / 1.05 /
+// 1 and the EDGE form 1.05 times as long.  Measured, ms, f32_block's choice in the plain form / the
+// rule's: 32768 samples of 5 x 4096, chi 16 185 / 100, 4 x 2048, chi 8 33.6 / 18.9, 2 x 4096, chi 2
+// 61 / 32, 6 x 4096, chi 32 319 / 165.
 struct F32Plan {
   int SB, NW;
   bool edge;
   size_t smem;
 };
 template <class Need, class Want>
-F32Plan f32_plan(int64_t total, int P, bool strong, int nsm, size_t max_smem, Need&& need, Want&& want) {
-  F32Plan p{f32_block(total, P, nsm), 0, strong, 0};
-  if (strong && p.SB == 8) p.SB = 4;
-  for (p.NW = want(p.SB); p.NW > 0; p.NW >>= 1) {
-    p.smem = need(p.SB, p.NW, p.edge);
-    if (p.smem <= max_smem) break;
-  }
-  return p;
+F32Plan f32_plan(int64_t total, int P, bool strong, int nsm, size_t max_smem, size_t smem_sm, Need&& need, Want&& want) {
+  auto form = [&](int SB, bool edge) {
+    F32Plan p{SB, 0, edge, 0};
+    for (p.NW = want(SB); p.NW > 0; p.NW >>= 1) {
+      p.smem = need(SB, p.NW, edge);
+      if (p.smem <= max_smem) break;
+    }
+    return p;
+  };
+  auto fit = [&](const F32Plan& p) { return smem_sm / (p.smem + 1024); };      // CTAs per SM by shared memory
+  const int block = f32_block(total, P, nsm);
+  F32Plan best = form(strong && block == 8 ? 4 : block, strong);
+  if (best.NW > 0 && fit(best) >= (size_t)f32_min_ctas(best.SB, f32_xbm(best.SB, P))) return best;
+  double least = 1e300;
+  for (int SB = block; SB > 0; SB >>= 1)
+    for (int edge = strong; edge < (SB < 8 ? 2 : 1); ++edge) {
+      const F32Plan p = form(SB, edge);
+      if (p.NW == 0) continue;
+      size_t ctas = fit(p);
+      const size_t regs = f32_min_ctas(SB, f32_xbm(SB, P));
+      ctas = ctas < 1 ? 1 : ctas > regs ? regs : ctas;
+      const int64_t wave = (int64_t)ctas * nsm * p.NW * 8 * SB;
+      const double t = (double)((total + wave - 1) / wave) * (SB == 8 ? 1.45 : SB == 4 ? 1.15 : SB == 2 ? 1.05 : 1.0) *
+                       (edge ? 1.05 : 1.0);
+      if (t < least) {
+        least = t;
+        best = p;
+      }
+    }
+  return best;
 }
 
 // Shared memory of a CTA that takes tiles of several lattices (P(i), Lx(i), i < n).  Each tile lays it

@@ -142,7 +142,7 @@ tnmc_status tnmc_launch_sample_simt(const tnmc_env* env, int precision, int64_t 
   const SampleArgs<float> a{d, d.K32, d.R32, d.fe32, B, seed, offset, spins_in, spins_out, logq, energy, flags, nullptr};
   const size_t stack = f32_stack_floats(d.P, d.Lx) * sizeof(float);
   const F32Plan p = f32_plan(
-      B, d.P, d.strong, nsm, (size_t)max_smem,
+      B, d.P, d.strong, nsm, (size_t)max_smem, (size_t)smem_sm,
       [&](int SB, int NW, bool edge) { return f32_smem(d.P, d.Lx, SB, NW, edge).total; },
       [&](int SB) {      // a CTA's stacks have to fit a fixed scratch
         int NW = 4;

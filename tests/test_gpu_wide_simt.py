@@ -74,3 +74,10 @@ def _check(precision, Ly, Lx, chi, sizes):
                                              (2, 4096, 2, (1, 700, 9001, 33000)), (6, 1100, 20, (2, 1500, 4001))])
 def test_f64_wide(Ly, Lx, chi, sizes):
     _check("f64", Ly, Lx, chi, sizes)
+
+
+@pytest.mark.parametrize("Ly,Lx,chi,sizes", [(2, 1300, 2, (3, 1500, 9001, 41000)), (4, 2048, 5, (5, 4000, 15001, 33000)),
+                                             (2, 4096, 2, (1, 1500, 9001, 66000)), (5, 3000, 13, (2, 1500, 4001, 41000)),
+                                             (6, 2100, 20, (2, 1500, 9001)), (7, 1200, 50, (2, 3100, 9001))])
+def test_f32_wide(Ly, Lx, chi, sizes):
+    _check("f32", Ly, Lx, chi, sizes)
