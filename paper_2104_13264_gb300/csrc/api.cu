@@ -86,28 +86,26 @@ bool is_integer_array(const double* p, size_t n) {
 // couplings in FP64, mean error of random configurations: 128 x 128 Gaussian couplings 3.0e-13 ->
 // 1.4e-13, with one field of 1e3 2.5e-12 -> 1.9e-13, of 1e6 2.1e-9 -> 0; 256 x 256 5.5e-13 -> 8.3e-13.
 int fixed_point_exponent(const tnmc_lattice& lat, size_t nJh, size_t nJv, size_t nh) {
-  double sum = 0.0;
-  int e0 = 0;      // magnitudes are taken relative to 2^e0: their sum cannot overflow
-  for (int pass = 0; pass < 2; ++pass) {
-    double mx = 0.0;
+  auto sum_of = [&](int shift) {      // of the magnitudes times 2^-shift
+    double s = 0.0;
     auto add = [&](const double* p, size_t n) {
-      for (size_t i = 0; i < n; ++i) {
-        if (pass == 0) mx = fmax(mx, fabs(p[i]));
-        else sum += ldexp(fabs(p[i]), -e0);
-      }
+      if (shift == 0)
+        for (size_t i = 0; i < n; ++i) s += fabs(p[i]);
+      else
+        for (size_t i = 0; i < n; ++i) s += ldexp(fabs(p[i]), -shift);
     };
     add(lat.Jh, nJh);
     add(lat.Jv, nJv);
     add(lat.h, nh);
-    if (pass == 0) {
-      if (mx == 0.0) return 0;
-      e0 = ilogb(mx);
-    }
-  }
-  const double terms = (double)(nJh + nJv + nh);
+    return s;
+  };
+  int e0 = 0;
+  double sum = sum_of(0);
+  if (sum == 0.0) return 0;
+  if (!isfinite(sum)) sum = sum_of(e0 = 64);
   int e = ilogb(sum) + 1;      // sum < 2^e
   // roundings of the couplings (half a unit each) and of `sum` itself
-  if (ldexp(sum, 63 - e) * (1.0 + 1e-7) + terms >= 0x1p63) ++e;
+  if (ldexp(sum, 63 - e) * (1.0 + 1e-7) + (double)(nJh + nJv + nh) >= 0x1p63) ++e;
   return e0 + e - 63;
 }
 
@@ -244,7 +242,13 @@ tnmc_status env_create(const tnmc_lattice* lat, double beta, int chi, int precis
     if (cnt == 0) return;
     memcpy(image.data() + o, src, cnt * 8);
     int64_t* q = reinterpret_cast<int64_t*>(image.data() + oq);
-    for (size_t i = 0; i < cnt; ++i) q[i] = llrint(ldexp(src[i], -d.qexp));
+    const int sh = -d.qexp;
+    if (sh >= -1000 && sh <= 1000) {      // times a power of two
+      const double unit = ldexp(1.0, sh);
+      for (size_t i = 0; i < cnt; ++i) q[i] = llrint(src[i] * unit);
+    } else {
+      for (size_t i = 0; i < cnt; ++i) q[i] = llrint(ldexp(src[i], sh));
+    }
   };
   put(lat->Jh, nJh, oJh, oqJh);
   put(lat->Jv, nJv, oJv, oqJv);
