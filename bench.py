@@ -551,7 +551,7 @@ def run_batched(args):
     else:
         peak, psrc = 1.25, "FP64 nominal 1.25 TFLOP/s"
     roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": round(achieved_tf, 3), "peak": round(peak, 3),
-            "frac": round(achieved_tf / peak, 5), "traffic": None, "kernel": "sample_batched_kernel",
+            "frac": round(achieved_tf / peak, 5), "traffic": None, "kernel": "sample_batched_%s_kernel" % prec,
             "kernel_ms": round(kern_s * 1e3, 3), "flop_per_launch": flops, "peak_source": psrc}
     step_ms = total_ms / args.steps
     acc_rate = n_accepted / (props * world * args.steps)

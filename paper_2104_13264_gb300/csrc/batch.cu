@@ -5,13 +5,13 @@
 // every instance in one launch.
 //
 // A plan fixes the instances, the proposals per instance B_i, the chains per
-// instance C, the precision (FP64 or FP32), the tile width NT and the order of
-// the work items.  One work item is one tile of NT samples of one instance;
+// instance C, the precision (FP64 or FP32), the samples per work item (`tile`) and the
+// order of the items.  One work item is `tile` consecutive samples of one instance;
 // the items sit in a device list (instance order, or longest-first by the
 // instance's per-sample cost) and a persistent grid of nSM x (CTAs per SM)
 // pulls them from an atomic counter, so that instances whose costs differ by
 // two orders of magnitude still fill the machine.  Each item runs the same
-// per-tile body as the single-instance SIMT sampler, so its outputs equal the
+// per-tile body as the single-instance sampler, so its outputs equal the
 // single-instance call at the same sample indices bit for bit.
 //
 // Sample indices: instance i at step k draws samples (i << 40) + k B_i + b;

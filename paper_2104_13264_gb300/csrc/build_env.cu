@@ -1158,12 +1158,7 @@ struct ShZ2 {
   int* flag;
 };
 
-// position of (a, k) in a doubled bond built from a bond of size D with e even states
-__device__ inline int dbl_idx(int a, int k, int D, int e) {
-  const bool odd = a >= e;
-  if (k == 0) return odd ? D + (a - e) : a;
-  return odd ? a : D + (D - e) + a;
-}
+// position l in a bond doubled from one of size D with e even states -> (a, k)
 __device__ inline void dbl_inv(int l, int D, int e, int& a, int& k) {
   if (l < D) {
     a = l;

@@ -15,8 +15,8 @@
 //     sum from the masks, and log q a product with integer exponents (one log per sample), so
 //     that nothing per site runs on the FP64 pipe.
 // Measured against one thread per sample (128 per CTA): 32 x 32, chi = 16, 65536 samples 11.3 ->
-// 4.88 ms (25 % of the FFMA peak; 1.7 warps per scheduler: latency, a third of it the ordered dot
-// product, draws and stores); 24 x 45, chi = 32, 16384 samples 28.8 -> 4.4 ms.
+// 4.8 ms (25 % of the FFMA peak; 1.7 warps per scheduler: latency, a third of it the ordered dot
+// product, draws and stores); 24 x 45, chi = 32, 16384 samples 28.8 -> 4.3 ms.
 //
 // The products and sums that decide a draw are taken in the order of a plain loop over the
 // bonds (the dot product <U[s], R> is passed from output lane to output lane), so the results

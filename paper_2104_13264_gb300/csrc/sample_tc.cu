@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
   float4* sR = reinterpret_cast<float4*>(sB + kStages * kStageBytes);        // [8][256]: each thread's R_{c+1}
   uint64_t* bars = reinterpret_cast<uint64_t*>(sB + kStages * kStageBytes + kRBytes);   // [0 .. kStages-1] tiles, [kStages] UMMA
   uint32_t* misc = reinterpret_cast<uint32_t*>(bars + kStages + 1);          // [0] tmem base, [1] abort, [2] tile ok
-  // thread 0's copy counter lives in shared memory (registers are the scarce resource):
-  // environment tiles whose copy was issued
+  // the producer's copy counter lives in shared memory, where the teardown reads it: environment tiles
+  // whose copy was issued
   int64_t* cnt = reinterpret_cast<int64_t*>(misc + 4);
   float* xw = reinterpret_cast<float*>(misc + 6);   // left steps: [2 halves][2][128] partial w(-), w(+)
   float* xmb = xw + 4 * kTile;                      // right steps: [step parity][2 halves][128] partial max
@@ -529,11 +529,11 @@ __global__ void __launch_bounds__(kThreads, 2) sample_tc_kernel(TcArgs a) {
   }
   // teardown (after the last step, or after a wait gave up): let the copies still in
   // flight land and the last committed UMMA finish (bounded waits with the full limit),
-  // then free TMEM.  The control thread observes the tile barriers in order and refills a stage
-  // only after a successful wait, so at most one phase of each is outstanding.
+  // then free TMEM.  The UMMA warp observes the tile barriers in order, and the producer warp refills a
+  // stage only in the step after its UMMA was waited for: at most one phase of each is outstanding.
   if (lead) {
-    // steps the control thread committed (g counts finished steps; an aborted step committed too),
-    // and tiles it saw land
+    // steps the UMMA warp committed (g counts finished steps; an aborted step committed too), and
+    // tiles it saw land
     const int64_t committed = g + (abort ? 1 : 0);
     const int64_t tiles_seen = g + ((abort && misc[2]) ? 1 : 0);
     for (int64_t q = tiles_seen; q < cnt[0]; ++q)
