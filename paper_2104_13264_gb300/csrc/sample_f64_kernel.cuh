@@ -13,7 +13,7 @@
 //     on rcp.approx and a residual step, clamps, maxima, draws and power-of-two scales are integer operations, and
 //     the energy is an exact 64-bit fixed-point sum.
 // Measured against one thread per sample (64 per CTA): 23 x 29, chi = 13, 5000 samples 26.2 ->
-// 5.9 ms (73 % of the FP64 pipe); 64 lattices 32 x 32, chi = 16 with 32 samples each 47.9 -> 6.0 ms.
+// 6.0 ms (76 % of the FP64 pipe); 64 lattices 32 x 32, chi = 16 with 32 samples each 47.9 -> 6.1 ms.
 //
 // A lane owns outputs x = g + LO i.  The dot product <U[s], R> goes through shared memory and is
 // summed over x = 0, 1, ... by one lane per (sample, spin): it is where the weights cancel, so
