@@ -10,8 +10,8 @@
 //     and tiles of down to 2 samples give an SM the warps that fill its FP64 pipe.
 //   - Scalar work (normalisation, draw) runs on one lane per sample; log q is a running
 //     product with an integer exponent (one log per sample), the division is two Newton steps
-//     on rcp.approx and a residual step, clamps, maxima, draws and power-of-two scales are integer operations, and
-//     the energy is an exact 64-bit fixed-point sum.
+//     on rcp.approx and a residual step, clamps, maxima, draws and power-of-two scales are
+//     integer operations, and the energy is an exact 64-bit fixed-point sum.
 // Measured against one thread per sample (64 per CTA): 23 x 29, chi = 13, 5000 samples 26.2 ->
 // 6.0 ms (76 % of the FP64 pipe); 64 lattices 32 x 32, chi = 16 with 32 samples each 47.9 -> 6.1 ms.
 //

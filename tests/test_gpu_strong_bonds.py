@@ -47,6 +47,27 @@ def test_f32_strong_bonds(Ly, Lx, chi, beta):
     env.free()
 
 
+def test_f32_batch_of_strong_and_weak_bonds():
+    """One strong lattice takes the whole plan to the other form, which leaves the weak ones' bits."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2104_13264_gb300 import binding as B
+    envs = [B.Env(*_lattice(6, 9, 48.0, 1), 48.0, 4, precisions=("f64", "f32")),
+            B.Env(*_lattice(7, 13, 2.0, 2), 2.0, 20, precisions=("f64", "f32"))]
+    for n in (60, 30000):
+        plan = B.Batch(envs, [n, n], chains=n // 2, precision="f32")
+        plan.set_step(5, 1)
+        out = plan.sample(plan.alloc_proposals())
+        for i, e in enumerate(envs):
+            ref = B.sample(e, n, seed=5, sample_offset=(i << 40) + n, precision="f32")
+            assert torch.equal(plan.view(out[0], i), ref[0])
+            for a, b in zip(out[1:], ref[1:]):
+                assert torch.equal(plan.rows(a, i), b)
+        plan.free()
+    for e in envs:
+        e.free()
+
+
 @pytest.mark.parametrize("beta", [19.0, 21.0, 32.0, 42.0])
 @pytest.mark.parametrize("Ly,Lx,chi", [(6, 9, 4), (7, 13, 20), (7, 14, 40)])
 def test_bf16_strong_bonds(Ly, Lx, chi, beta):
