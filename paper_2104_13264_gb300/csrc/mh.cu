@@ -294,12 +294,12 @@ __global__ void __launch_bounds__(32 * kScanWarps)
 // Decisions are those of the sequential rule.  tnmc_mh_step of one chain of 10^4 proposals takes
 // 414 us with one warp and 71 us with one CTA (bands, scan, copy and launches), 64 chains of 1024
 // 63 and 31 us.
-constexpr int kCtaBlock = 4096;
+constexpr int kCtaBlock = 4096, kCtaMinBlock = 512;
 constexpr int kCtaChunk = 32;
 constexpr int kCtaLook = 8;
 constexpr int kCtaThreads = 128;
 // A CTA takes a few thousand cycles whatever T is, a warp about 83 per proposal: worth it from
-// T = 256 on (2048 chains of 128: 46.7 us against 46.0), while the CTAs of all chains fit the SMs in a few waves.
+// T = 256 on (2048 chains of 128: 46.7 us against 46.0), up to 2048 chains (of 8192: 2.1 ms against 2.3).
 constexpr int64_t kCtaMinT = 256, kCtaMaxChains = 2048;
 
 inline __host__ __device__ size_t mh_cta_smem(int nb) {
@@ -509,7 +509,17 @@ tnmc_status tnmc_launch_mh_core(int64_t n, double beta, const tnmc::Allocator& a
   TNMC_CUDA_TRY(cudaGetLastError());
   const int threads = 128;   // 4 warps: the warp form's shared-memory layout
   if (C <= kCtaMaxChains && T >= kCtaMinT) {   // one CTA per chain
-    const int nb = T < kCtaBlock ? (int)((T + kCtaChunk - 1) / kCtaChunk) * kCtaChunk : kCtaBlock;
+    // The largest block of proposals that leaves all chains' CTAs resident at once: a long block has
+    // fewer serial steps per proposal, but CTAs that wait for an SM cost more.  ms, 4096 in every case / now /
+    // one warp per chain: 256 x 8192 0.49 / 0.42 / 0.65, 600 x 8192 1.02 / 0.74 / 0.92, 2048 x 4096
+    // 1.67 / 1.14 / 1.23.
+    int dev = 0, nsm = 0, smem_sm = 0;
+    TNMC_CUDA_TRY(cudaGetDevice(&dev));
+    TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    TNMC_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    int nb = T < kCtaBlock ? (int)((T + kCtaChunk - 1) / kCtaChunk) * kCtaChunk : kCtaBlock;
+    while (nb > kCtaMinBlock && C > (int64_t)nsm * (smem_sm / (int)(mh_cta_smem(nb) + 2048)))
+      nb = nb / 2 > kCtaMinBlock ? (nb / 2 + kCtaChunk - 1) / kCtaChunk * kCtaChunk : kCtaMinBlock;
     const size_t smem = mh_cta_smem(nb);
     TNMC_CUDA_TRY(cudaFuncSetAttribute(mh_scan_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     mh_scan_cta_kernel<<<(unsigned)C, kCtaThreads, smem, stream>>>(T, nb, beta, seed, step_offset, prop_logq,
