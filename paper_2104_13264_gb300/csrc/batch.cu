@@ -68,34 +68,43 @@ __device__ __forceinline__ uint64_t global_ns() {
 
 // cta_ns[2 i], cta_ns[2 i + 1]: when CTA i started and when it found no item left (global
 // timer, ns): the load balance of the launch is sum(busy) / (grid x makespan).
-// FP32: a CTA of NW warps takes an item at a time, NW 8 SB samples at once.
+//
+// FP32: a CTA of NW warps takes NW 8 SB samples at a time.  A work item of `tile` samples is handed out
+// in parts of that size (consecutive counter values), so that small batches, whose blocks are small,
+// spread over the SMs: 4 lattices of 12 to 20 columns, chi 4, 512 samples each 2.13 -> 0.58 ms.
 template <int SB, int XBM, bool EDGE>
 __global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM))
     sample_batched_f32_kernel(const SampleArgs<float>* __restrict__ tab, const int2* __restrict__ items, int64_t nitems,
                               int tile, unsigned long long* counter, float* scratch, size_t stack_elems,
                               uint64_t* cta_ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int2 item;
+  __shared__ int inst;
+  __shared__ int64_t base;
   __shared__ SampleArgs<float> a;
-  const int step = (blockDim.x >> 5) * (8 * SB);
+  const int step = (blockDim.x >> 5) * (8 * SB), per = tile / step;
   float* stack = scratch + (size_t)blockIdx.x * stack_elems * step;
   if (threadIdx.x == 0) cta_ns[2 * blockIdx.x] = global_ns();
   for (;;) {
     if (threadIdx.x == 0) {
       const unsigned long long k = atomicAdd(counter, 1ull);
-      item = (k < (unsigned long long)nitems) ? items[k] : make_int2(-1, -1);
+      inst = -1;
+      if (k < (unsigned long long)nitems * per) {
+        const int2 it = items[k / per];
+        inst = it.x;
+        base = (int64_t)it.y * tile + (int64_t)(k % per) * step;
+      }
     }
     __syncthreads();
-    const int2 it = item;
+    const int i = inst;
+    const int64_t base0 = base;
     __syncthreads();
-    if (it.x < 0) break;
+    if (i < 0) break;
     {
-      const int* src = reinterpret_cast<const int*>(tab + it.x);
+      const int* src = reinterpret_cast<const int*>(tab + i);
       for (int q = threadIdx.x; q < (int)(sizeof(a) / sizeof(int)); q += blockDim.x) reinterpret_cast<int*>(&a)[q] = src[q];
     }
     __syncthreads();
-    for (int64_t base = (int64_t)it.y * tile; base < (int64_t)(it.y + 1) * tile && base < a.B; base += step)
-      sample_f32_tile<SB, XBM, EDGE>(a, base, smem_raw, stack);
+    if (base0 < a.B) sample_f32_tile<SB, XBM, EDGE>(a, base0, smem_raw, stack);
   }
   if (threadIdx.x == 0) cta_ns[2 * blockIdx.x + 1] = global_ns();
 }
@@ -369,7 +378,7 @@ tnmc_status plan_setup(tnmc_batch* p, int max_Lx) {
     if (st != TNMC_OK) return st;
     p->s_warp[q] = S;
     p->warps[q] = NW;
-    const int64_t unit = f64 ? S : p->tile;
+    const int64_t unit = (int64_t)S * NW;
     for (int i = 0; i < p->n; ++i) tiles += ((q ? p->chains : p->B[i]) + unit - 1) / unit;
     grid = std::max(grid, std::min<int64_t>(tiles, (int64_t)nsm * std::max(per_sm, 1)));
     samples = std::max(samples, (size_t)S * NW);
