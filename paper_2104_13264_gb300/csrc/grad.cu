@@ -692,6 +692,10 @@ tnmc_status tnmc_launch_logq_grad(const tnmc_env* env, int64_t B, const int8_t* 
   TNMC_CUDA_TRY(cudaGetDevice(&dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   TNMC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  // small bonds, large batches (P = 4: from about 9700 samples, P = 8: from 39000): one thread per
+  // sample, measured on both sides in grad_small.cu
+  if (d.P <= 8 && B >= (int64_t)(d.P == 4 ? 64 : 256) * nsm && tnmc_grad_small_smem(d.Lx, d.P) <= (size_t)max_optin)
+    return tnmc_launch_logq_grad_small(env, B, spins, weights, grad, nsm, stream);
   const bool staged = !d.strong && grad_smem(d.P, d.Lx, true).total <= (size_t)max_optin;
   const size_t smem = grad_smem(d.P, d.Lx, staged).total;
   if (smem > (size_t)max_optin) {

@@ -83,8 +83,8 @@ def test_bf16_strong_bonds(Ly, Lx, chi, beta):
 
 
 @pytest.mark.parametrize("beta", [19.0, 21.0, 32.0, 42.0])
-@pytest.mark.parametrize("Ly,Lx,chi", [(6, 9, 4), (7, 13, 20), (7, 14, 40)])
-def test_grad_strong_bonds(Ly, Lx, chi, beta):
+@pytest.mark.parametrize("Ly,Lx,chi,n", [(6, 9, 4, 40), (7, 13, 20, 40), (7, 14, 40, 40), (6, 9, 4, 10000)])
+def test_grad_strong_bonds(Ly, Lx, chi, n, beta):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2104_13264_gb300 import binding as B
@@ -96,8 +96,8 @@ def test_grad_strong_bonds(Ly, Lx, chi, beta):
     ref = tnmc.Env(Lx, Ly, beta, chi, Jh, Jv, h)
     ref.M = [[ex["tensors"][r, c, :bd[r, c], :, :bd[r, c + 1]].astype(np.float32).astype(np.float64)
               for c in range(Lx)] for r in range(Ly)]
-    sp = B.sample(env, 40, seed=7)[0].cpu().numpy()
-    w = np.random.default_rng(chi).random(40)
+    sp = B.sample(env, n, seed=7)[0].cpu().numpy()
+    w = np.random.default_rng(chi).random(n)
     _, G = tnmc.logq_grad(ref, sp, w)
     grad = B.logq_backward(env, torch.from_numpy(sp).cuda(), torch.from_numpy(w).float().cuda())
     g = grad.cpu().numpy().reshape(Ly, Lx, P, 2, P)
