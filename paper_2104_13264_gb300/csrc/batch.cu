@@ -71,7 +71,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 //
 // FP32: a CTA of NW warps takes NW 8 SB samples at a time.  A work item of `tile` samples is handed out
 // in parts of that size (consecutive counter values), so that small batches, whose blocks are small,
-// spread over the SMs: 4 lattices of 12 to 20 columns, chi 4, 512 samples each 2.13 -> 0.58 ms.
+// spread over the SMs: 4 lattices of 12 to 20 columns, chi 4, 512 samples each 2.13 -> 0.55 ms.
 template <int SB, int XBM, bool EDGE>
 __global__ void __launch_bounds__(128, f32_min_ctas(SB, XBM))
     sample_batched_f32_kernel(const SampleArgs<float>* __restrict__ tab, const int2* __restrict__ items, int64_t nitems,

@@ -146,26 +146,26 @@ __device__ __forceinline__ bool usable_scale3(T& s) {
   return false;
 }
 
-// sel[0..k) = the k <= m rows of largest norm (descending; ties by index).  A NaN norm becomes zero
-// (returns false): it compares false with everything, and the ranks have to be a permutation.
+// sel[0..k) = the k <= m <= 64 rows of largest norm (descending; ties by index).  A NaN norm compares
+// false with everything and leaves ranks unset: such norms then count as zero (returns false).
 template <typename T, typename VJ>
 __device__ bool select_rows(VJ d, int m, int k, int* sel) {
-  bool ok = true;
-  for (int i = 0; i < m; ++i)
-    if (!(d[i] >= 0)) {
-      d[i] = T(0);
-      ok = false;
+  for (bool clean = true;; clean = false) {
+    unsigned long long seen = 0;
+    for (int i = 0; i < m; ++i) {
+      int rank = 0;
+      const T di = d[i];
+      for (int j = 0; j < m; ++j) {
+        const T dj = d[j];
+        rank += (dj > di) || (dj == di && j < i);
+      }
+      if (rank < k) sel[rank] = i;
+      seen |= 1ull << rank;
     }
-  for (int i = 0; i < m; ++i) {
-    int rank = 0;
-    const T di = d[i];
-    for (int j = 0; j < m; ++j) {
-      const T dj = d[j];
-      rank += (dj > di) || (dj == di && j < i);
-    }
-    if (rank < k) sel[rank] = i;
+    if (!clean || (~seen & ((1ull << k) - 1)) == 0) return clean;
+    for (int i = 0; i < m; ++i)
+      if (!(d[i] >= 0)) d[i] = T(0);
   }
-  return ok;
 }
 
 // Successive SVD of an MPS of ns sites (site i at M.at(i * cap), layout [dl][p][dr]):
